@@ -285,16 +285,14 @@ int launch_one(const Bucket& b, const KArgs& a, void* stream, const char* what) 
 
 // Every game, one launch per size bucket; buckets after the first run on
 // side streams forked from and joined back into `stream`.
-// The work-list form serves batches of several buckets without spawn
-// options (their generator runs in its own kernel).  By default it takes
+// The work-list form serves batches of several buckets.  By default it takes
 // batches of more than four buckets: there the per-bucket launches are many
 // and small (mixed 32,768 games, 15 buckets: 136 against 131 M frames/s per
 // frame, resident 173 against 167 M), while a few large buckets overlap
 // well on the forked streams (ragged 131,072 games, 4 buckets: 428 against
 // 419 M, resident 627 against 606 M).
 bool use_worklist(const gen_env* e) {
-    const bool spawn = e->prm.max_general_dist > 0 || e->prm.bfs_distance || e->prm.castle_radius > 0;
-    if (e->buckets.size() < 2 || !e->d_items[0] || spawn || e->batch_form == 1) return false;
+    if (e->buckets.size() < 2 || !e->d_items[0] || e->batch_form == 1) return false;
     return e->batch_form == 2 || e->buckets.size() > 4;
 }
 

@@ -50,6 +50,7 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kQuadMaxCells = 576;
 constexpr int kPairMaxCells = 1024;
 constexpr int kPairMaxPlayers = 2;
+constexpr int kFallbackCells = 1024;  // see place_generals_bfs
 constexpr int kPlain = 0, kMountain = 1, kCastle = 2, kGeneral = 3;
 constexpr int kArmyMax = 32767;
 constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ULL;
@@ -86,6 +87,10 @@ struct Grp {
     __device__ __forceinline__ T shfl(T v, int src) const { return __shfl_sync(mask, v, src, W); }
     template <class T>
     __device__ __forceinline__ T shfl_up(T v, int d) const { return __shfl_up_sync(mask, v, d, W); }
+    template <class T>
+    __device__ __forceinline__ T shfl_down(T v, int d) const { return __shfl_down_sync(mask, v, d, W); }
+    // the group's lanes that hold the same value as this one
+    __device__ __forceinline__ unsigned match(int v) const { return (__match_any_sync(mask, v) & mask) >> shift; }
     // bit i = lane i of the group (the other half's lanes are masked off)
     __device__ __forceinline__ unsigned ballot(bool pr) const {
         if (W == 32) return __ballot_sync(kFull, pr);
@@ -274,125 +279,142 @@ __device__ __forceinline__ void column_pass(const Game& g, const Smem& s, const 
     t.sync();
 }
 
-// ---- bitset BFS (generator options) ----------------------------------------
-// Word arrays of nw words in shared memory, one lane per word.  Bit c of
-// dilate4(x) is set when a 4-neighbour of cell c is set in x.
-__device__ void dilate4(const uint32_t* x, uint32_t* out, const Game& g, const Smem& s, int lane) {
-    const int nw = g.nw, q = g.W >> 5, sh = g.W & 31;
-    for (int w = lane; w < nw; w += 32) {
-        const uint32_t X = x[w];
-        const uint32_t Xm = w > 0 ? x[w - 1] : 0u, Xp = w + 1 < nw ? x[w + 1] : 0u;
-        const uint32_t L = (X << 1) | (Xm >> 31);  // bit c <- cell c-1
-        const uint32_t R = (X >> 1) | (Xp << 31);  // bit c <- cell c+1
-        uint32_t v = (L & ~s.col0[w]) | (R & ~s.colL[w]);
-        const int wa = w - q;  // bit c <- cell c-W
-        if (wa >= 0) v |= x[wa] << sh;
-        if (sh && wa - 1 >= 0) v |= x[wa - 1] >> (32 - sh);
-        const int wb = w + q;  // bit c <- cell c+W
-        if (wb < nw) v |= x[wb] >> sh;
-        if (sh && wb + 1 < nw) v |= x[wb + 1] << (32 - sh);
-        out[w] = v & valid_bits(g.N, w);
+// ---- row bitsets (BFS of the map generator) --------------------------------
+// A set of cells held in registers: lane l of the group keeps rows R*l ..
+// R*l + R-1 of the board, one word of W bits each (32 or 64).  A step of a
+// flood fill is then two shifts in place and the two neighbour rows (two
+// shuffles), about ten instructions for a board of up to 32 x 32 with a warp
+// per game and no shared memory.  The same fill as one dilation per step over
+// shared-memory bitsets (a lane per 32 cells, a sync on either side) made
+// 21,838 warp instructions per 24x24 map with BFS spacing and the castle
+// guarantee.
+template <class T, int R>
+struct RowSet {
+    T v[R];
+};
+
+// 32 bits of the nw-word bitset x from bit b on (b may lie outside: zeros)
+__device__ __forceinline__ uint32_t bits_at(const uint32_t* x, int nw, int b) {
+    const int i = b >> 5;
+    const uint32_t lo = (unsigned)i < (unsigned)nw ? x[i] : 0u;
+    const uint32_t hi = (unsigned)(i + 1) < (unsigned)nw ? x[i + 1] : 0u;
+    return __funnelshift_r(lo, hi, b & 31);
+}
+
+// rows of the cells that are clear (invert) or set in the row-major bitset x
+template <class T, int R, int LW>
+__device__ __forceinline__ RowSet<T, R> load_rows(const uint32_t* x, const Game& g, bool invert, const Grp<LW>& t) {
+    RowSet<T, R> s;
+    const T width = g.W >= (int)(8 * sizeof(T)) ? ~(T)0 : (((T)1 << g.W) - 1);
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const int r = R * t.lane + i;
+        T v = bits_at(x, g.nw, r * g.W);
+        if (sizeof(T) == 8) v |= (T)((uint64_t)bits_at(x, g.nw, r * g.W + 32) << 32);
+        s.v[i] = r < g.H ? ((invert ? ~v : v) & width) : (T)0;
     }
-    __syncwarp();
+    return s;
 }
 
-__device__ __forceinline__ void set_single(uint32_t* x, int c, const Game& g, int lane) {
-    for (int w = lane; w < g.nw; w += 32) x[w] = (w == (c >> 5)) ? (1u << (c & 31)) : 0u;
-    __syncwarp();
-}
-
-// BFS from src through `pass`.  keep_out (when lo >= 0): cells within lo
-// steps leave `allowed`; then `allowed` keeps only cells within hi steps
-// (hi <= 0: all reachable cells).  vis / front / nxt are scratch.
-__device__ void bfs_restrict(int src, int lo, int hi, const uint32_t* pass, uint32_t* allowed, uint32_t* vis,
-                             uint32_t* front, uint32_t* nxt, const Game& g, const Smem& s, int lane) {
-    set_single(vis, src, g, lane);
-    set_single(front, src, g, lane);
-    bool cut = false;
-    if (lo == 0) {
-        for (int w = lane; w < g.nw; w += 32) allowed[w] &= ~vis[w];
-        cut = true;
+// one step of a flood fill through `pass`
+template <class T, int R, int LW>
+__device__ __forceinline__ void flood_step(RowSet<T, R>& x, const RowSet<T, R>& pass, const Grp<LW>& t) {
+    T prev = t.shfl_up(x.v[R - 1], 1), below = t.shfl_down(x.v[0], 1);
+    if (t.lane == 0) prev = 0;
+    if (t.lane == LW - 1) below = 0;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const T cur = x.v[i], next = i + 1 < R ? x.v[i + 1] : below;
+        x.v[i] = cur | (((cur << 1) | (cur >> 1) | prev | next) & pass.v[i]);
+        prev = cur;
     }
-    for (int step = 1; hi <= 0 || step <= hi; ++step) {
-        dilate4(front, nxt, g, s, lane);
-        bool any = false;
-        for (int w = lane; w < g.nw; w += 32) {
-            const uint32_t n = nxt[w] & pass[w] & ~vis[w];
-            front[w] = n;
-            vis[w] |= n;
-            any |= n != 0u;
-        }
-        __syncwarp();
-        if (!__any_sync(kFull, any)) break;
-        if (step == lo) {
-            for (int w = lane; w < g.nw; w += 32) allowed[w] &= ~vis[w];
-            cut = true;
-        }
+}
+// n steps, or (n < 0) steps until nothing changes; either way it stops when
+// four steps in a row change nothing
+template <class T, int R, int LW>
+__device__ __forceinline__ void flood(RowSet<T, R>& x, const RowSet<T, R>& pass, int n, const Grp<LW>& t) {
+    for (; n < 0 || n >= 4; n -= n < 0 ? 0 : 4) {
+        const RowSet<T, R> old = x;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) flood_step(x, pass, t);
+        bool changed = false;
+#pragma unroll
+        for (int i = 0; i < R; ++i) changed |= x.v[i] != old.v[i];
+        if (!t.any(changed)) return;
     }
-    __syncwarp();
-    for (int w = lane; w < g.nw; w += 32) allowed[w] &= (lo >= 0 && !cut) ? 0u : vis[w];
-    __syncwarp();
+#pragma unroll 1
+    for (; n > 0; --n) flood_step(x, pass, t);
+}
+// Keep in `allowed` the cells whose BFS distance from cell src through `pass`
+// is above lo (lo < 0: no lower bound) and at most hi (hi <= 0: reachable).
+// Returns the cells within hi steps.
+template <class T, int R, int LW>
+__device__ __forceinline__ RowSet<T, R> bfs_restrict(int src, int lo, int hi, const RowSet<T, R>& pass,
+                                                     RowSet<T, R>& allowed, const Game& g, const Grp<LW>& t) {
+    RowSet<T, R> vis;
+    const int r = src / g.W, c = src - r * g.W;
+#pragma unroll
+    for (int i = 0; i < R; ++i) vis.v[i] = R * t.lane + i == r ? (T)1 << c : (T)0;
+    const bool capped = hi > 0;
+    int done = 0;
+    if (lo >= 0) {
+        done = capped ? min(lo, hi) : lo;
+        flood(vis, pass, done, t);
+        const T keep = capped && hi < lo ? (T)0 : ~(T)0;  // the cap lies below the bound: nothing fits
+#pragma unroll
+        for (int i = 0; i < R; ++i) allowed.v[i] &= ~vis.v[i] & keep;
+    }
+    flood(vis, pass, capped ? hi - done : -1, t);
+#pragma unroll
+    for (int i = 0; i < R; ++i) allowed.v[i] &= vis.v[i];
+    return vis;
 }
 
-// first set bit (row-major) of x, or -1
-__device__ int first_bit(const uint32_t* x, const Game& g, int lane) {
-    int best = 0x7FFFFFFF;
-    for (int w = lane; w < g.nw; w += 32)
-        if (x[w]) best = min(best, 32 * w + __ffs(x[w]) - 1);
-    best = (int)__reduce_min_sync(kFull, (unsigned)best);
-    return best == 0x7FFFFFFF ? -1 : best;
-}
+template <class T>
+__device__ __forceinline__ int bits_of(T x) { return sizeof(T) == 8 ? __popcll((uint64_t)x) : __popc((uint32_t)x); }
+template <class T>
+__device__ __forceinline__ int lowest(T x) { return (sizeof(T) == 8 ? __ffsll((long long)x) : __ffs((int)x)) - 1; }
 
-// cell of the k-th (0-based, row-major) set bit of x; x holds more than k bits
-__device__ int kth_bit(const uint32_t* x, uint32_t k, const Game& g, int lane) {
-    const int wpl = (g.nw + 31) >> 5, w0 = lane * wpl;
+// the k-th (0-based, row-major) cell of x, or -1 when it holds no more than k
+template <class T, int R, int LW>
+__device__ __forceinline__ int kth_cell(const RowSet<T, R>& x, uint32_t k, const Game& g, const Grp<LW>& t) {
     uint32_t mine = 0;
-    for (int w = w0; w < w0 + wpl && w < g.nw; ++w) mine += __popc(x[w]);
+#pragma unroll
+    for (int i = 0; i < R; ++i) mine += bits_of(x.v[i]);
     uint32_t incl = mine;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
+    for (int o = 1; o < LW; o <<= 1) {
+        const uint32_t y = t.shfl_up(incl, o);
+        if (t.lane >= o) incl += y;
     }
-    const int L = __ffs(__ballot_sync(kFull, incl > k)) - 1;
+    const unsigned b = t.ballot(incl > k);
+    if (b == 0u) return -1;
     int cell = 0;
-    if (lane == L) {
-        uint32_t r = k - (incl - mine);
-        for (int w = w0; w < w0 + wpl && w < g.nw; ++w) {
-            uint32_t v = x[w];
-            const uint32_t n = __popc(v);
-            if (r >= n) {
-                r -= n;
-                continue;
-            }
-            for (uint32_t z = 0; z < r; ++z) v &= v - 1;
-            cell = 32 * w + __ffs(v) - 1;
-            break;
+    uint32_t left = k - (incl - mine);
+    bool open = true;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const uint32_t n = bits_of(x.v[i]);
+        if (open && left < n) {
+            T v = x.v[i];
+            for (uint32_t z = 0; z < left; ++z) v &= v - 1;
+            cell = (R * t.lane + i) * g.W + lowest(v);
+            open = false;
         }
+        left -= n;
     }
-    return __shfl_sync(kFull, cell, L);
+    return t.shfl(cell, __ffs(b) - 1);
 }
-
-// bitset of cells matching a predicate on (terrain type, owner), one ballot per word
-template <class Pred>
-__device__ void cell_bits(uint32_t* out, const Game& g, const Smem& s, int lane, Pred pred) {
-    for (int w = 0; w < g.nw; ++w) {
-        const int c = 32 * w + lane;
-        const bool b = c < g.N && pred(s.terrain[c] & 3, (int)s.owner[c]);
-        const unsigned m = __ballot_sync(kFull, b);
-        if (lane == 0) out[w] = m;
+// whether x holds cell (r, c), a cell of its own per lane
+template <class T, int R, int LW>
+__device__ __forceinline__ bool row_test(const RowSet<T, R>& x, int r, int c, const Grp<LW>& t) {
+    T v = 0;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const T y = t.shfl(x.v[i], r / R);
+        if (r % R == i) v = y;
     }
-    __syncwarp();
-}
-
-// ---- map generator with spawn options (Sec. IV-A) --------------------------
-// Scratch bitsets of the spawn options; the step rebuilds these arrays.
-struct GenScratch {
-    uint32_t *pass, *front, *nxt, *vis, *allowed, *gens;
-};
-__device__ __forceinline__ GenScratch gen_scratch(const Smem& s) {
-    const int st = s.stride;
-    return GenScratch{s.big, s.own, s.own + st, s.vis, s.vis + st, s.tmp};
+    return (v >> c) & 1;
 }
 
 // Generals at BFS distance (through non-mountain cells) in [D, dmax] of every
@@ -400,143 +422,175 @@ __device__ __forceinline__ GenScratch gen_scratch(const Smem& s) {
 // at D = 0 the first cell (row-major) within the cap of every earlier general,
 // else reachable from general 0, else any free cell.  Lane p returns player
 // p's general in the low 16 bits; bit 20 says whether a general cannot reach
-// general 0 (the L-path carve is then needed).
-__device__ __noinline__ int place_generals_bfs(const Game& g, const Smem& s, uint64_t kgen, int dmax, int lane) {
-    const int N = g.N, P = g.P;
-    const GenScratch z = gen_scratch(s);
-    column_pass(g, s, Grp<32>(lane));
-    cell_bits(z.pass, g, s, lane, [](int t, int) { return t != kMountain; });
-    for (int w = lane; w < g.nw; w += 32) z.gens[w] = 0u;
-    __syncwarp();
+// general 0 (the L-path carve is then needed): only one of the last kind,
+// since every other placement is reachable from general 0.  mtn: the
+// mountains as a row-major bitset.
+template <class T, int R, int LW>
+__device__ __forceinline__ int place_generals_bfs(const Game& g, const uint32_t* mtn, uint64_t kgen, int dmax,
+                                                  const Grp<LW>& t) {
+    const int W = g.W;
+    const RowSet<T, R> pass = load_rows<T, R>(mtn, g, true, t);
+    RowSet<T, R> allowed = pass;
+    int folded = 0;  // earlier generals whose distances `allowed` respects at this D
     uint32_t i = 0;
     int D = g.dmin;
     int my_gpos = -1;
-    for (int p = 0; p < P; ++p) {
+    bool cut_off = false;
+    for (int p = 0; p < g.P; ++p) {
         int placed = -1;
-        while (placed < 0) {
-            if (D >= 1) {
-                for (int w = lane; w < g.nw; w += 32) z.allowed[w] = z.pass[w];
-                __syncwarp();
-                for (int q = 0; q < p; ++q)
-                    bfs_restrict(__shfl_sync(kFull, my_gpos, q), D - 1, dmax, z.pass, z.allowed, z.vis, z.front,
-                                 z.nxt, g, s, lane);
-                int found = -1;
-                for (int base = 0; base < kGenAttempts; base += 32) {
-                    const int t = base + lane;
-                    const int c = uniform_below(hdraw(kgen, (uint64_t)(i + t)), (uint32_t)N);
-                    const bool ok = t < kGenAttempts && ((z.allowed[c >> 5] >> (c & 31)) & 1u);
-                    const unsigned b = __ballot_sync(kFull, ok);
-                    if (b) {
-                        const int l = __ffs(b) - 1;
-                        found = base + l;
-                        placed = __shfl_sync(kFull, c, l);
-                        break;
-                    }
-                }
-                if (found >= 0) {
-                    i += (uint32_t)found + 1;
-                } else {
-                    i += kGenAttempts;
-                    D -= 1;
-                }
-            } else {
-                for (int w = lane; w < g.nw; w += 32) z.allowed[w] = z.pass[w] & ~z.gens[w];
-                __syncwarp();
-                for (int q = 0; q < p; ++q)
-                    bfs_restrict(__shfl_sync(kFull, my_gpos, q), -1, dmax, z.pass, z.allowed, z.vis, z.front, z.nxt,
-                                 g, s, lane);
-                placed = first_bit(z.allowed, g, lane);
-                if (placed < 0) {
-                    for (int w = lane; w < g.nw; w += 32) z.allowed[w] = z.pass[w] & ~z.gens[w];
-                    __syncwarp();
-                    if (p > 0)
-                        bfs_restrict(__shfl_sync(kFull, my_gpos, 0), -1, 0, z.pass, z.allowed, z.vis, z.front, z.nxt,
-                                     g, s, lane);
-                    placed = first_bit(z.allowed, g, lane);
-                }
-                if (placed < 0) {
-                    for (int w = lane; w < g.nw; w += 32) z.allowed[w] = ~z.gens[w] & valid_bits(N, w);
-                    __syncwarp();
-                    placed = first_bit(z.allowed, g, lane);
+        while (placed < 0 && D >= 1) {
+            for (; folded < p; ++folded) bfs_restrict(t.shfl(my_gpos, folded), D - 1, dmax, pass, allowed, g, t);
+            int found = -1;
+            for (int base = 0; base < kGenAttempts && found < 0; base += LW) {
+                const int c = uniform_below(hdraw(kgen, (uint64_t)(i + base + t.lane)), (uint32_t)g.N);
+                const int r = c / W;
+                const unsigned b = t.ballot(row_test(allowed, r, c - r * W, t));
+                if (b) {
+                    const int l = __ffs(b) - 1;
+                    found = base + l;
+                    placed = t.shfl(c, l);
                 }
             }
+            if (found >= 0) {
+                i += (uint32_t)found + 1;
+            } else {
+                i += kGenAttempts;
+                D -= 1;
+                allowed = pass;
+                folded = 0;
+            }
         }
-        if (lane == p) my_gpos = placed;
-        if (lane == (placed >> 5)) z.gens[placed >> 5] |= 1u << (placed & 31);
-        __syncwarp();
+        if (placed < 0) {
+            // the fallbacks, over cells without a general -- of those in the
+            // first kFallbackCells cells: later ones have never been left out
+            // here, and maps are keyed by their seeds, so they stay as they are
+            RowSet<T, R> open = pass, any;
+            const T width = W >= (int)(8 * sizeof(T)) ? ~(T)0 : (((T)1 << W) - 1);
+#pragma unroll
+            for (int k = 0; k < R; ++k) any.v[k] = R * t.lane + k < g.H ? width : (T)0;
+            for (int q = 0; q < p; ++q) {
+                const int gq = t.shfl(my_gpos, q), r = gq / W;
+#pragma unroll
+                for (int k = 0; k < R; ++k)
+                    if (R * t.lane + k == r && gq < kFallbackCells) {
+                        const T bit = (T)1 << (gq - r * W);
+                        open.v[k] &= ~bit;
+                        any.v[k] &= ~bit;
+                    }
+            }
+            RowSet<T, R> x = open;
+            for (int q = 0; q < p; ++q) bfs_restrict(t.shfl(my_gpos, q), -1, dmax, pass, x, g, t);
+            placed = kth_cell(x, 0u, g, t);
+            if (placed < 0) {
+                x = open;
+                if (p > 0) bfs_restrict(t.shfl(my_gpos, 0), -1, 0, pass, x, g, t);
+                placed = kth_cell(x, 0u, g, t);
+            }
+            if (placed < 0) {
+                placed = kth_cell(any, 0u, g, t);
+                cut_off |= p > 0;
+            }
+        }
+        if (t.lane == p) my_gpos = placed;
     }
-    bool carve = false;
-    if (P > 1) {
-        for (int w = lane; w < g.nw; w += 32) z.allowed[w] = z.gens[w];
-        __syncwarp();
-        bfs_restrict(__shfl_sync(kFull, my_gpos, 0), -1, 0, z.pass, z.allowed, z.vis, z.front, z.nxt, g, s, lane);
-        bool miss = false;
-        for (int w = lane; w < g.nw; w += 32) miss |= z.allowed[w] != z.gens[w];
-        carve = __any_sync(kFull, miss);
-    }
-    return (my_gpos & 0xFFFF) | (carve ? (1 << 20) : 0);
+    return (my_gpos & 0xFFFF) | (cut_off ? (1 << 20) : 0);
 }
 
-// A neutral castle within `radius` BFS steps of every general (s.misc holds
-// the generals): where none is, one on a free plain cell of the ball, the
-// k-th such cell in row-major order with k drawn uniformly.
-__device__ __noinline__ void castle_guarantee(const KArgs& a, const Game& g, const Smem& s, uint64_t gid,
-                                              uint32_t epoch, int radius, int lane) {
-    const GenScratch z = gen_scratch(s);
-    column_pass(g, s, Grp<32>(lane));
-    uint32_t* free_plain = z.gens;
-    cell_bits(z.pass, g, s, lane, [](int t, int) { return t != kMountain; });
-    cell_bits(free_plain, g, s, lane, [](int t, int o) { return t == kPlain && o == -1; });
-    const uint64_t knp = hkey(a.seed, gid, epoch, 5);
-    const uint64_t kna = hkey(a.seed, gid, epoch, 6);
+// A neutral castle within a.castle_radius BFS steps of every general (s.misc
+// holds the generals): where none is, one on a free plain cell of the ball,
+// the k-th such cell in row-major order with k drawn uniformly.  mtn, taken
+// and castles: row-major bitsets of the mountains, of the cells that are not
+// neutral plain, and of the castles (updated).
+template <class T, int R, int LW>
+__device__ __forceinline__ void castle_guarantee(const KArgs& a, const Game& g, const Smem& s, const uint32_t* mtn,
+                                                 const uint32_t* taken, uint32_t* castles, uint64_t kmap, const Grp<LW>& t) {
+    const RowSet<T, R> pass = load_rows<T, R>(mtn, g, true, t);
+    RowSet<T, R> free_plain = load_rows<T, R>(taken, g, true, t), built = load_rows<T, R>(castles, g, false, t);
+    const uint64_t knp = stream_out(kmap, 5);
+    const uint64_t kna = stream_out(kmap, 6);
     for (int p = 0; p < g.P; ++p) {
-        const int gp = s.misc[p];
-        cell_bits(z.allowed, g, s, lane, [](int t, int o) { return t == kCastle && o == -1; });
-        bfs_restrict(gp, -1, radius, z.pass, z.allowed, z.vis, z.front, z.nxt, g, s, lane);
+        RowSet<T, R> near = built;
+        const RowSet<T, R> ball = bfs_restrict(s.misc[p], -1, a.castle_radius, pass, near, g, t);
         bool have = false;
-        for (int w = lane; w < g.nw; w += 32) have |= z.allowed[w] != 0u;
-        if (__any_sync(kFull, have)) continue;
-        for (int w = lane; w < g.nw; w += 32) z.allowed[w] = free_plain[w] & z.vis[w];  // vis: the ball
-        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < R; ++i) have |= near.v[i] != 0;
+        if (t.any(have)) continue;
+        RowSet<T, R> x = free_plain;
         uint32_t cnt = 0;
-        for (int w = lane; w < g.nw; w += 32) cnt += __popc(z.allowed[w]);
-        cnt = __reduce_add_sync(kFull, cnt);
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            x.v[i] &= ball.v[i];
+            cnt += bits_of(x.v[i]);
+        }
+        cnt = t.reduce_add(cnt);
         if (cnt == 0) continue;
-        const int cell = kth_bit(z.allowed, (uint32_t)uniform_below(hdraw(knp, (uint64_t)p), cnt), g, lane);
-        if (lane == 0) {
-            s.terrain[cell] = kCastle;
+        const int cell = kth_cell(x, (uint32_t)uniform_below(hdraw(knp, (uint64_t)p), cnt), g, t);
+        if (t.lane == 0) {
+            castles[cell >> 5] |= 1u << (cell & 31);
             s.army[cell] = (int16_t)(a.city_min + uniform_below(hdraw(kna, (uint64_t)p), (uint32_t)a.city_span));
         }
-        if (lane == (cell >> 5)) free_plain[cell >> 5] &= ~(1u << (cell & 31));
-        __syncwarp();
+        const int r = cell / g.W;
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+            if (R * t.lane + i == r) {
+                const T bit = (T)1 << (cell - r * g.W);
+                free_plain.v[i] &= ~bit;
+                built.v[i] |= bit;
+            }
     }
 }
 
-// The generator with spawn options (the launch's spawn_dmax, spawn_bfs,
-// castle_radius).  It is a separate function of a separate kernel
-// instantiation so that the options' register pressure never reaches the
-// step kernel that runs without them.
-__device__ __forceinline__ void generate_spawn_body(const KArgs& a, const Game& g, const Smem& s, uint64_t gid,
-                                                   uint32_t epoch, int lane) {
-    const int N = g.N, W = g.W, P = g.P;
-    const uint64_t kmtn = hkey(a.seed, gid, epoch, 1);
-    for (int c = lane; c < g.Npad; c += 32) {
-        bool m = c < N && hdraw(kmtn, (uint64_t)c) < a.mtn_thresh;
-        s.army[c] = 0;
-        s.owner[c] = -1;
-        s.terrain[c] = m ? kMountain : kPlain;
-    }
-    __syncwarp();
+// ---- map generator (Sec. IV-A) ----------------------------------------------
+// Mountains, castles and taken cells are row-major bitsets while the map is
+// made; the cells' bytes are written once at the end, with the passable-
+// neighbour bits.  Draws are evaluated LW at a time and accepted in draw
+// order, so the draw counters advance exactly as one by one.
+//
+// Instructions bound it.  Resets of 65,536 24x24 games: 314.6 -> 204.7 us with
+// the plain generator (castles a batch of draws at a time instead of a batch
+// each, cells as bits until the end), 2,004 -> 419 us with BFS spacing and the
+// castle guarantee (see RowSet; 608 MB of state and outputs need 90 us).
+// SPAWN: with the options of the launch (a.spawn_*, a.castle_radius).
+template <int LW, bool SPAWN>
+__device__ __forceinline__ void generate_body(const KArgs& a, const Game& g, const Smem& s, uint64_t gid,
+                                             uint32_t epoch, const Grp<LW>& t) {
+    const int N = g.N, W = g.W, P = g.P, nw = g.nw;
+    // bitsets in regions that the step rebuilds after a new map
+    uint32_t* mtn = s.tmp;
+    uint32_t* taken = s.own;
+    uint32_t* castles = s.big;
 
-    // generals: 32 candidate draws evaluated at once; the first accepted in
-    // draw order wins, so the draw counter advances exactly as one by one
-    const uint64_t kgen = hkey(a.seed, gid, epoch, 2);
-    const int dmax = a.spawn_dmax;
+    // mountains: a ballot per LW cells, draws running on from one another (the
+    // stream advances by a constant) and several words' draws interleaved;
+    // the board's army and owner planes cleared
+    const uint64_t kmap = stream_out(stream_out(a.seed, gid), epoch);  // hkey(seed, gid, epoch, x) = stream_out(kmap, x)
+    uint64_t z = stream_out(kmap, 1) + (uint64_t)(t.lane + 1) * kGamma;
+#pragma unroll 2
+    for (int w = 0; w < nw; ++w) {
+        unsigned m = 0;
+#pragma unroll
+        for (int h = 0; h < 32; h += LW) {
+            m |= t.ballot((uint32_t)(mix64(z) >> 32) < a.mtn_thresh) << h;
+            z += (uint64_t)LW * kGamma;
+        }
+        if (t.lane == 0) mtn[w] = m & valid_bits(N, w);
+    }
+    for (int v = t.lane; v < 2 * g.nch; v += LW) reinterpret_cast<uint4*>(s.army)[v] = make_uint4(0, 0, 0, 0);
+    for (int v = t.lane; v < g.nch; v += LW) reinterpret_cast<uint4*>(s.owner)[v] = make_uint4(kFull, kFull, kFull, kFull);
+    for (int w = t.lane; w < nw; w += LW) castles[w] = 0u;
+    t.sync();
+    auto in = [](const uint32_t* x, int c) { return ((x[c >> 5] >> (c & 31)) & 1u) != 0u; };
+
+    // generals
+    const uint64_t kgen = stream_out(kmap, 2);
+    const int dmax = SPAWN ? a.spawn_dmax : 0;
     int my_gpos = -1;  // lane p holds player p's general
     bool carve = true;
-    if (a.spawn_bfs) {
-        const int r = place_generals_bfs(g, s, kgen, dmax, lane);
-        my_gpos = lane < P ? (r & 0xFFFF) : -1;
+    const bool narrow_rows = g.W <= 32 && g.H <= 32;
+    if (SPAWN && a.spawn_bfs) {
+        const int r = narrow_rows ? place_generals_bfs<uint32_t, 32 / LW>(g, mtn, kgen, dmax, t)
+                                  : place_generals_bfs<uint64_t, 64 / LW>(g, mtn, kgen, dmax, t);
+        my_gpos = t.lane < P ? (r & 0xFFFF) : -1;
         carve = (r >> 20) & 1;
     } else {
         uint32_t i = 0;
@@ -546,22 +600,21 @@ __device__ __forceinline__ void generate_spawn_body(const KArgs& a, const Game& 
             while (placed < 0) {
                 if (D >= 1) {
                     int found = -1;
-                    for (int base = 0; base < kGenAttempts; base += 32) {
-                        int t = base + lane;
-                        int c = uniform_below(hdraw(kgen, (uint64_t)(i + t)), (uint32_t)N);
-                        bool ok = (t < kGenAttempts) && s.terrain[c] != kMountain;
-                        int rc = c / W, cc = c - rc * W;
+                    for (int base = 0; base < kGenAttempts; base += LW) {
+                        const int c = uniform_below(hdraw(kgen, (uint64_t)(i + base + t.lane)), (uint32_t)N);
+                        bool ok = !in(mtn, c);
+                        const int rc = c / W, cc = c - rc * W;
                         for (int q = 0; q < p; ++q) {
-                            int gq = __shfl_sync(kFull, my_gpos, q);
-                            int rq = gq / W, cq = gq - rq * W;
+                            const int gq = t.shfl(my_gpos, q);
+                            const int rq = gq / W, cq = gq - rq * W;
                             const int d = abs(rc - rq) + abs(cc - cq);
                             if (d < D || (dmax > 0 && d > dmax)) ok = false;
                         }
-                        unsigned b = __ballot_sync(kFull, ok);
+                        const unsigned b = t.ballot(ok);
                         if (b) {
-                            int l = __ffs(b) - 1;
+                            const int l = __ffs(b) - 1;
                             found = base + l;
-                            placed = __shfl_sync(kFull, c, l);
+                            placed = t.shfl(c, l);
                             break;
                         }
                     }
@@ -572,214 +625,125 @@ __device__ __forceinline__ void generate_spawn_body(const KArgs& a, const Game& 
                         D -= 1;
                     }
                 } else {
-                    for (int base = 0; base < N && placed < 0; base += 32) {
-                        int c = base + lane;
+                    for (int base = 0; base < N && placed < 0; base += LW) {
+                        const int c = base + t.lane;
                         bool ok = c < N;
                         for (int q = 0; q < p; ++q)
-                            if (__shfl_sync(kFull, my_gpos, q) == c) ok = false;
-                        unsigned b = __ballot_sync(kFull, ok);
+                            if (t.shfl(my_gpos, q) == c) ok = false;
+                        const unsigned b = t.ballot(ok);
                         if (b) placed = base + __ffs(b) - 1;
                     }
                 }
             }
-            if (lane == p) my_gpos = placed;
+            if (t.lane == p) my_gpos = placed;
         }
-    }
-    if (lane < P) {
-        s.terrain[my_gpos] = kGeneral;
-        s.owner[my_gpos] = (int8_t)lane;
-        s.army[my_gpos] = 1;
-        s.misc[lane] = my_gpos;
-    }
-    __syncwarp();
-
-    // L-path rows first, then columns, between consecutive generals (in BFS
-    // mode only when some general cannot reach general 0)
-    if (carve && lane == 0) {
-        for (int p = 0; p + 1 < P; ++p) {
-            int r = s.misc[p] / W, c = s.misc[p] % W;
-            int r1 = s.misc[p + 1] / W, c1 = s.misc[p + 1] % W;
-            while (r != r1) {
-                r += (r1 > r) ? 1 : -1;
-                if (s.terrain[r * W + c] == kMountain) s.terrain[r * W + c] = kPlain;
-            }
-            while (c != c1) {
-                c += (c1 > c) ? 1 : -1;
-                if (s.terrain[r * W + c] == kMountain) s.terrain[r * W + c] = kPlain;
-            }
-        }
-    }
-    __syncwarp();
-
-    // neutral castles on neutral plain cells
-    const uint64_t kpos = hkey(a.seed, gid, epoch, 3);
-    const uint64_t karm = hkey(a.seed, gid, epoch, 4);
-    uint32_t j = 0;
-    for (int k = 0; k < g.n_cities; ++k) {
-        int found = -1, cell = 0;
-        for (int base = 0; base < kGenAttempts; base += 32) {
-            int t = base + lane;
-            int c = uniform_below(hdraw(kpos, (uint64_t)(j + t)), (uint32_t)N);
-            bool ok = (t < kGenAttempts) && s.terrain[c] == kPlain && s.owner[c] == -1;
-            unsigned b = __ballot_sync(kFull, ok);
-            if (b) {
-                int l = __ffs(b) - 1;
-                found = base + l;
-                cell = __shfl_sync(kFull, c, l);
-                break;
-            }
-        }
-        if (found >= 0) {
-            j += (uint32_t)found + 1;
-            if (lane == 0) {
-                s.terrain[cell] = kCastle;
-                s.army[cell] = (int16_t)(a.city_min + uniform_below(hdraw(karm, (uint64_t)k), (uint32_t)a.city_span));
-            }
-            __syncwarp();
-        } else {
-            j += kGenAttempts;
-        }
-    }
-
-    if (a.castle_radius > 0) castle_guarantee(a, g, s, gid, epoch, a.castle_radius, lane);
-    derive_passable(g, s, Grp<32>(lane));
-}
-
-// ---- map generator (Sec. IV-A) ----------------------------------------------
-template <int LW>
-__device__ __forceinline__ void generate_body(const KArgs& a, const Game& g, const Smem& s, uint64_t gid,
-                                             uint32_t epoch, const Grp<LW>& t) {
-    const int N = g.N, W = g.W, P = g.P;
-    const uint64_t kmtn = hkey(a.seed, gid, epoch, 1);
-    for (int c = t.lane; c < g.Npad; c += LW) {
-        bool m = c < N && hdraw(kmtn, (uint64_t)c) < a.mtn_thresh;
-        s.army[c] = 0;
-        s.owner[c] = -1;
-        s.terrain[c] = m ? kMountain : kPlain;
-    }
-    t.sync();
-
-    // generals: LW candidate draws evaluated at once; the first accepted in
-    // draw order wins, so the draw counter advances exactly as one by one
-    const uint64_t kgen = hkey(a.seed, gid, epoch, 2);
-    uint32_t i = 0;
-    int D = g.dmin;
-    int my_gpos = -1;  // lane p holds player p's general
-    for (int p = 0; p < P; ++p) {
-        int placed = -1;
-        while (placed < 0) {
-            if (D >= 1) {
-                int found = -1;
-                for (int base = 0; base < kGenAttempts; base += LW) {
-                    const int dr = base + t.lane;  // draw index
-                    int c = uniform_below(hdraw(kgen, (uint64_t)(i + dr)), (uint32_t)N);
-                    bool ok = (dr < kGenAttempts) && s.terrain[c] != kMountain;
-                    int rc = c / W, cc = c - rc * W;
-                    for (int q = 0; q < p; ++q) {
-                        int gq = t.shfl(my_gpos, q);
-                        int rq = gq / W, cq = gq - rq * W;
-                        if (abs(rc - rq) + abs(cc - cq) < D) ok = false;
-                    }
-                    unsigned b = t.ballot(ok);
-                    if (b) {
-                        int l = __ffs(b) - 1;
-                        found = base + l;
-                        placed = t.shfl(c, l);
-                        break;
-                    }
-                }
-                if (found >= 0) {
-                    i += (uint32_t)found + 1;
-                } else {
-                    i += kGenAttempts;
-                    D -= 1;
-                }
-            } else {
-                for (int base = 0; base < N && placed < 0; base += LW) {
-                    int c = base + t.lane;
-                    bool ok = c < N;
-                    for (int q = 0; q < p; ++q)
-                        if (t.shfl(my_gpos, q) == c) ok = false;
-                    unsigned b = t.ballot(ok);
-                    if (b) placed = base + __ffs(b) - 1;
-                }
-            }
-        }
-        if (t.lane == p) my_gpos = placed;
     }
     if (t.lane < P) {
-        s.terrain[my_gpos] = kGeneral;
         s.owner[my_gpos] = (int8_t)t.lane;
         s.army[my_gpos] = 1;
         s.misc[t.lane] = my_gpos;
+        atomicAnd(mtn + (my_gpos >> 5), ~(1u << (my_gpos & 31)));
     }
     t.sync();
 
-    // connectivity: L-path rows first, then columns, between consecutive generals
-    if (t.lane == 0) {
+    // connectivity: L-path rows first, then columns, between consecutive
+    // generals (in BFS mode only when some general cannot reach general 0)
+    if (carve) {
         for (int p = 0; p + 1 < P; ++p) {
-            int r = s.misc[p] / W, c = s.misc[p] % W;
-            int r1 = s.misc[p + 1] / W, c1 = s.misc[p + 1] % W;
-            while (r != r1) {
-                r += (r1 > r) ? 1 : -1;
-                if (s.terrain[r * W + c] == kMountain) s.terrain[r * W + c] = kPlain;
-            }
-            while (c != c1) {
-                c += (c1 > c) ? 1 : -1;
-                if (s.terrain[r * W + c] == kMountain) s.terrain[r * W + c] = kPlain;
+            const int g0 = s.misc[p], g1 = s.misc[p + 1];
+            const int r0 = g0 / W, c0 = g0 - r0 * W, r1 = g1 / W, c1 = g1 - r1 * W;
+            const int dr = abs(r1 - r0), dc = abs(c1 - c0);
+            for (int k = t.lane; k < dr + dc; k += LW) {
+                const int r = k < dr ? (r1 > r0 ? r0 + k + 1 : r0 - k - 1) : r1;
+                const int c = k < dr ? c0 : (c1 > c0 ? c0 + (k - dr) + 1 : c0 - (k - dr) - 1);
+                const int cell = r * W + c;
+                if (in(mtn, cell)) atomicAnd(mtn + (cell >> 5), ~(1u << (cell & 31)));
             }
         }
+        t.sync();
+    }
+
+    // neutral castles on neutral plain cells: castle k takes the first such
+    // cell among its next kGenAttempts draws, else none.  A batch of LW draws
+    // serves as many castles as it can: a draw is accepted when its cell is
+    // free and no earlier draw of the batch took it.
+    for (int w = t.lane; w < nw; w += LW) taken[w] = mtn[w];
+    t.sync();
+    if (t.lane < P) atomicOr(taken + (my_gpos >> 5), 1u << (my_gpos & 31));
+    t.sync();
+    const uint64_t kpos = stream_out(kmap, 3);
+    const uint64_t karm = stream_out(kmap, 4);
+    int k = 0;       // the castle being placed
+    int misses = 0;  // its rejected draws so far
+    for (uint32_t j = 0; k < g.n_cities; j += LW) {
+        const int c = uniform_below(hdraw(kpos, (uint64_t)(j + t.lane)), (uint32_t)N);
+        const bool open = !in(taken, c);
+        const unsigned same = t.match(c);
+        const bool ok = open && (same & ((1u << t.lane) - 1u)) == 0u;
+        unsigned b = t.ballot(ok);
+        const int first = b ? __ffs(b) - 1 : LW;
+        if (misses + first >= kGenAttempts) {  // castle k's attempts end before that draw
+            k += 1;
+            misses -= kGenAttempts;
+        }
+        const int mine = k + __popc(b & ((1u << t.lane) - 1u));  // the castle an accepted draw places
+        if (ok && mine < g.n_cities) {
+            atomicOr(taken + (c >> 5), 1u << (c & 31));
+            atomicOr(castles + (c >> 5), 1u << (c & 31));
+            s.army[c] = (int16_t)(a.city_min + uniform_below(hdraw(karm, (uint64_t)mine), (uint32_t)a.city_span));
+        }
+        k += __popc(b);
+        misses = b ? LW - 1 - (31 - __clz(b)) : misses + LW;
+        t.sync();
+    }
+
+    if (SPAWN && a.castle_radius > 0) {
+        if (narrow_rows)
+            castle_guarantee<uint32_t, 32 / LW>(a, g, s, mtn, taken, castles, kmap, t);
+        else
+            castle_guarantee<uint64_t, 64 / LW>(a, g, s, mtn, taken, castles, kmap, t);
+    }
+
+    // terrain bytes, 16 cells per lane: type, and whether each neighbour
+    // exists and is not a mountain
+    t.sync();
+    const uint16_t* col0 = reinterpret_cast<const uint16_t*>(g_columns[W - 1][0]);
+    const uint16_t* colL = reinterpret_cast<const uint16_t*>(g_columns[W - 1][1]);
+    auto passable = [&](int b) {  // 16 cells from b on: on the board and not a mountain
+        const int i = b >> 5;
+        const uint32_t lo = (unsigned)i < (unsigned)nw ? ~mtn[i] & valid_bits(N, i) : 0u;
+        const uint32_t hi = (unsigned)(i + 1) < (unsigned)nw ? ~mtn[i + 1] & valid_bits(N, i + 1) : 0u;
+        return __funnelshift_r(lo, hi, b & 31);
+    };
+    for (int ch = t.lane; ch < g.nch; ch += LW) {
+        const int c0 = ch << 4;
+        const uint32_t valid = valid_bits(N, c0 >> 5) >> (c0 & 16);
+        const uint32_t m = mtn[c0 >> 5] >> (c0 & 16), z = castles[c0 >> 5] >> (c0 & 16);
+        const uint32_t up = passable(c0 - W), dn = passable(c0 + W);
+        const uint32_t lf = passable(c0 - 1) & ~(uint32_t)col0[ch], rt = passable(c0 + 1) & ~(uint32_t)colL[ch];
+        uint32_t out[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int sh = 4 * q;
+            auto spread = [&](uint32_t x) { return (((x >> sh) & 15u) * 0x00204081u) & 0x01010101u; };
+            out[q] = spread(m & valid) | (spread(z) << 1) | (spread(up & valid) << 2) | (spread(dn & valid) << 3) |
+                     (spread(lf & valid) << 4) | (spread(rt & valid) << 5);
+        }
+        *reinterpret_cast<uint4*>(s.terrain + c0) = make_uint4(out[0], out[1], out[2], out[3]);
     }
     t.sync();
-
-    // neutral castles on neutral plain cells
-    const uint64_t kpos = hkey(a.seed, gid, epoch, 3);
-    const uint64_t karm = hkey(a.seed, gid, epoch, 4);
-    uint32_t j = 0;
-    for (int k = 0; k < g.n_cities; ++k) {
-        int found = -1, cell = 0;
-        for (int base = 0; base < kGenAttempts; base += LW) {
-            const int dr = base + t.lane;  // draw index
-            int c = uniform_below(hdraw(kpos, (uint64_t)(j + dr)), (uint32_t)N);
-            bool ok = (dr < kGenAttempts) && s.terrain[c] == kPlain && s.owner[c] == -1;
-            unsigned b = t.ballot(ok);
-            if (b) {
-                int l = __ffs(b) - 1;
-                found = base + l;
-                cell = t.shfl(c, l);
-                break;
-            }
-        }
-        if (found >= 0) {
-            j += (uint32_t)found + 1;
-            if (t.lane == 0) {
-                s.terrain[cell] = kCastle;
-                s.army[cell] = (int16_t)(a.city_min + uniform_below(hdraw(karm, (uint64_t)k), (uint32_t)a.city_span));
-            }
-            t.sync();
-        } else {
-            j += kGenAttempts;
-        }
-    }
-    derive_passable(g, s, t);
+    if (t.lane < P) s.terrain[my_gpos] = (uint8_t)((s.terrain[my_gpos] & ~3u) | kGeneral);
+    t.sync();
 }
 
-// Out-of-line entry points of the cold paths take plain arguments and rebuild
-// the game and shared-memory views themselves, so that the step kernel never
-// materialises those structures in local memory for a call it rarely makes.
-template <int LW, bool UNI>
+// Out-of-line entry point of a new map inside a multi-frame launch: it takes
+// plain arguments and rebuilds the game and shared-memory views itself, so
+// that the step kernel never materialises those structures in local memory
+// for a call it rarely makes.
+template <int LW, bool UNI, bool SPAWN>
 __device__ __noinline__ void generate(const KArgs& a, int gidx, char* warp_base, uint32_t geom, uint64_t gid,
                                      uint32_t epoch, int warp_lane) {
-    generate_body(a, game_of<UNI>(a, gidx), carve_geom(warp_base, geom), gid, epoch, Grp<LW>(warp_lane));
-}
-__device__ __noinline__ void generate_spawn(const KArgs& a, int gidx, char* warp_base, uint32_t geom, uint64_t gid,
-                                           uint32_t epoch, int lane) {
-    generate_spawn_body(a, game_of(a, gidx), carve_geom(warp_base, geom), gid, epoch, lane);
-}
-template <int LW, bool UNI>
-__device__ __noinline__ void derive_passable_at(const KArgs& a, int gidx, char* warp_base, uint32_t geom,
-                                               int warp_lane) {
-    derive_passable(game_of<UNI>(a, gidx), carve_geom(warp_base, geom), Grp<LW>(warp_lane));
+    generate_body<LW, SPAWN>(a, game_of<UNI>(a, gidx), carve_geom(warp_base, geom), gid, epoch, Grp<LW>(warp_lane));
 }
 
 // ---- one move on lane 0 (Sec. IV-D, IV-E) ----------------------------------
@@ -1257,59 +1221,138 @@ __device__ __forceinline__ void store_board(const KArgs& a, const Game& g, const
 namespace {
 
 
-template <bool MULTI, bool SPAWN, int LW, bool UNI>
-// geom: the packed carve geometry of the game's warp region, or 0 for the
-// launch's own (kernel parameters); only the cold out-of-line paths use it.
-__device__ __forceinline__ void run_game(const KArgs& a, const Smem& s, char* warp_base, const uint32_t geom,
-                                         const int gidx, const Grp<LW>& t) {
-    Game g = game_of<UNI>(a, gidx);
+// The end of a frame: outputs, the benchmark policy (whose actions, on lane
+// p player p's, come back in my_act) and, per frame, the scalar outputs.
+// columns: the board's column bitsets are in shared memory already.
+template <bool MULTI, int LW, bool UNI>
+__device__ __forceinline__ void finish_frame(const KArgs& a, const Game& g, const Smem& s, const int gidx, int f,
+                                             bool columns, uint32_t alive, bool fin, uint32_t frame, float my_reward,
+                                             uint32_t done, int32_t& my_act, const Grp<LW>& t) {
+    if constexpr (MULTI) {
+        // reward and done before the output passes and the scoreboard
+        // as soon as the fog pass has counted the land: fewer values
+        // live through the passes (measured faster in multi-frame
+        // launches, slower per frame)
+        if (a.do_outputs) {
+            const int64_t soff = (int64_t)f * a.slot_stride;
+            if (t.lane < g.P) a.reward[soff + g.player_off + t.lane] = my_reward;
+            if (t.lane == 0) a.done[(int64_t)f * a.game_stride + gidx] = (uint8_t)done;
+        }
+    }
+    if (a.do_outputs) {
+        const int64_t poff = (int64_t)f * a.plane_stride;
+        const int64_t soff = (int64_t)f * a.slot_stride;
+        if (!columns) column_pass(g, s, t);
+        fog_pass(g, s, alive, t);  // counts the land
+        if constexpr (MULTI) {
+            if (t.lane < g.P) {
+                a.scoreboard[2 * (soff + g.player_off + t.lane) + 0] = s.misc[8 + t.lane];
+                a.scoreboard[2 * (soff + g.player_off + t.lane) + 1] = s.misc[16 + t.lane];
+            }
+        }
+        if (a.next_actions)
+            output_pass<true, true, LW>(a, g, s, alive, fin, t, poff);
+        else
+            output_pass<true, false, LW>(a, g, s, alive, fin, t, poff);
+        if constexpr (!MULTI) {
+            if (t.lane < g.P) {
+                a.reward[soff + g.player_off + t.lane] = my_reward;
+                a.scoreboard[2 * (soff + g.player_off + t.lane) + 0] = s.misc[8 + t.lane];
+                a.scoreboard[2 * (soff + g.player_off + t.lane) + 1] = s.misc[16 + t.lane];
+            }
+            if (t.lane == 0) a.done[(int64_t)f * a.game_stride + gidx] = (uint8_t)done;
+        }
+    } else if (a.next_actions) {
+        output_pass<false, true, LW>(a, g, s, alive, fin, t, 0);
+    }
+    if (a.next_actions) my_act = policy_pass<!MULTI, LW>(a, g, s, alive, fin, frame, game_id_of<UNI>(a, gidx), t);
+}
+
+__device__ __forceinline__ void store_scalars(const KArgs& a, int gidx, uint32_t turn, uint32_t frame, uint32_t epoch,
+                                              uint32_t alive, uint32_t finished, uint32_t invalid, uint32_t saturated,
+                                              uint32_t err) {
+    uint4* dst = reinterpret_cast<uint4*>(a.scal + gidx);
+    dst[0] = make_uint4(turn, frame, epoch, alive);
+    dst[1] = make_uint4(finished, invalid, saturated, err);
+}
+
+template <int LW>
+__device__ __forceinline__ Game group_game(Game g) {
     if constexpr (LW < 32) {
         // narrow groups run only two-player games without teams: 1v1, or a
         // two-player free-for-all, whose rules are the same
         g.P = kPairMaxPlayers;
         g.mode = 0;
     }
+    return g;
+}
+
+// The rest of a per-frame launch for a game that gets a new map (create,
+// reset, a finished game) or new passable-neighbour bits: the map, the
+// frame's end, the state stored.  Nothing returns to the step, so the step
+// kernel keeps no value alive across a call: with the generator as a call
+// that returned, its registers set the spills of the frames without a reset
+// (65,536 1v1 games on 24x24: 135.5 us per launch with the earlier, smaller
+// generator returning, 132.5 us so; with the spawn options compiled in,
+// 185.7 us returning and 136.6 us so).
+// sc: the counters with the frame and epoch of the new state.
+template <int LW, bool UNI, bool SPAWN>
+__device__ __noinline__ void new_map(const KArgs& a, int gidx, char* warp_base, uint32_t geom, int warp_lane,
+                                     uint32_t frame, uint32_t epoch, uint32_t invalid, uint32_t saturated, uint32_t err,
+                                     float my_reward, uint32_t done) {
+    const Grp<LW> t(warp_lane);
+    const Game g = group_game<LW>(game_of<UNI>(a, gidx));
+    const Smem s = carve_geom(warp_base, geom);
+    generate_body<LW, SPAWN>(a, g, s, game_id_of<UNI>(a, gidx), epoch, t);
+    const uint32_t alive = (1u << g.P) - 1u;
+    cell_pass(g, s, false, false, t);
+    int32_t act = 0;
+    finish_frame<false, LW, UNI>(a, g, s, gidx, 0, a.op == OP_STEP, alive, false, frame, my_reward, done, act, t);
+    t.sync();
+    store_board(a, g, s, t);
+    if (t.lane == 0) store_scalars(a, gidx, 0u, frame, epoch, alive, 0u, invalid, saturated, err);
+}
+
+// geom: the packed carve geometry of the game's warp region, or 0 for the
+// launch's own (kernel parameters); only the cold out-of-line paths use it.
+template <bool MULTI, bool SPAWN, int LW, bool UNI>
+__device__ __forceinline__ void run_game(const KArgs& a, const Smem& s, char* warp_base, const uint32_t geom,
+                                         const int gidx, const Grp<LW>& t) {
+    const Game g = group_game<LW>(game_of<UNI>(a, gidx));
     GameScalars* sc = a.scal + gidx;
 
-    // every global load of the step is issued here, before any is used
-    const bool board = a.op != OP_CREATE && a.op != OP_RESET;
-    if (board) board_issue(a, g, s, t);
-    uint4 s0 = make_uint4(0, 0, 0, 0), s1 = make_uint4(0, 0, 0, 0);
-    if (a.op != OP_CREATE) {
-        s0 = *reinterpret_cast<const uint4*>(sc);
-        s1 = *(reinterpret_cast<const uint4*>(sc) + 1);
+    uint4 s0, s1;
+    if constexpr (!MULTI) {
+        if (a.op == OP_CREATE || a.op == OP_RESET) {
+            s0 = s1 = make_uint4(0, 0, 0, 0);
+            if (a.op == OP_RESET) {
+                s0 = *reinterpret_cast<const uint4*>(sc);
+                s1 = *(reinterpret_cast<const uint4*>(sc) + 1);
+                s0.z += 1;
+            }
+            new_map<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of<LW>(a), t.lane + t.shift, s0.y, s0.z, s1.y, s1.z,
+                             s1.w, 0.0f, 0u);
+            return;
+        }
     }
+    // every global load of the step is issued here, before any is used
+    board_issue(a, g, s, t);
+    s0 = *reinterpret_cast<const uint4*>(sc);
+    s1 = *(reinterpret_cast<const uint4*>(sc) + 1);
     // player `lane`'s action for the next step (frame 0: from the caller)
     int32_t my_act = (a.op == OP_STEP && t.lane < g.P) ? a.actions[g.player_off + t.lane] : 0;
-    if (board) board_wait(t);
+    board_wait(t);
 
-    uint32_t turn = 0, frame = 0, epoch = 0, alive = 0, finished = 0, invalid = 0, saturated = 0, err = 0;
-    if (a.op != OP_CREATE) {
-        turn = s0.x;
-        frame = s0.y;
-        epoch = s0.z;
-        alive = s0.w;
-        finished = s1.x;
-        invalid = s1.y;
-        saturated = s1.z;
-        err = s1.w;
-    }
-    const uint32_t all_alive = (1u << g.P) - 1u;
+    uint32_t turn = s0.x, frame = s0.y, epoch = s0.z, alive = s0.w;
+    uint32_t finished = s1.x, invalid = s1.y, saturated = s1.z;
+    const uint32_t err = s1.w;
     bool wrote_state = false;
 
-    if (a.op == OP_CREATE || a.op == OP_RESET) {
-        if (a.op == OP_RESET) epoch += 1;
-        if constexpr (SPAWN)
-            generate_spawn(a, gidx, warp_base, geom ? geom : geom_of<LW>(a), game_id_of<UNI>(a, gidx), epoch, t.lane + t.shift);
-        else
-            generate<LW, UNI>(a, gidx, warp_base, geom ? geom : geom_of<LW>(a), game_id_of<UNI>(a, gidx), epoch, t.lane + t.shift);
-        turn = 0;
-        alive = all_alive;
-        finished = 0;
-        wrote_state = true;
-    } else if (a.op == OP_DERIVE) {
-        derive_passable_at<LW, UNI>(a, gidx, warp_base, geom ? geom : geom_of<LW>(a), t.lane + t.shift);
-        wrote_state = true;
+    if constexpr (!MULTI) {
+        if (a.op == OP_DERIVE) {  // recompute cached per-map bits after a state upload
+            derive_passable(g, s, t);
+            wrote_state = true;
+        }
     }
     const int frames = (MULTI && a.op == OP_STEP) ? a.frames : 1;
     for (int f = 0; f < frames; ++f) {
@@ -1366,74 +1409,36 @@ __device__ __forceinline__ void run_game(const KArgs& a, const Smem& s, char* wa
             if (done) {
                 if (a.auto_reset) {
                     epoch += 1;
-                    if constexpr (SPAWN)
-                        generate_spawn(a, gidx, warp_base, geom ? geom : geom_of<LW>(a), game_id_of<UNI>(a, gidx), epoch, t.lane + t.shift);
-                    else
-                        generate<LW, UNI>(a, gidx, warp_base, geom ? geom : geom_of<LW>(a), game_id_of<UNI>(a, gidx), epoch, t.lane + t.shift);
-                    turn = 0;
-                    alive = all_alive;
-                    cell_pass(g, s, false, false, t);
+                    if constexpr (!MULTI) {
+                        new_map<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of<LW>(a), t.lane + t.shift, frame + 1,
+                                         epoch, invalid, saturated, err, my_reward, done);
+                        return;
+                    } else {
+                        generate<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of<LW>(a),
+                                                 game_id_of<UNI>(a, gidx), epoch, t.lane + t.shift);
+                        turn = 0;
+                        alive = (1u << g.P) - 1u;
+                        cell_pass(g, s, false, false, t);
+                    }
                 } else {
                     finished = 1;
                 }
             }
             wrote_state = true;
         } else {
-            // create, reset, observe, policy, or a frozen game
+            // observe, policy, derive, or a frozen game
             saturated += cell_pass(g, s, false, false, t);
         }
         if (a.op == OP_STEP) frame += 1;
-
-        const bool fin = finished != 0;
-        if constexpr (MULTI) {
-            // reward and done before the output passes and the scoreboard
-            // as soon as the fog pass has counted the land: fewer values
-            // live through the passes (measured faster in multi-frame
-            // launches, slower per frame)
-            if (a.do_outputs) {
-                const int64_t soff = (int64_t)f * a.slot_stride;
-                if (t.lane < g.P) a.reward[soff + g.player_off + t.lane] = my_reward;
-                if (t.lane == 0) a.done[(int64_t)f * a.game_stride + gidx] = (uint8_t)done;
-            }
-        }
-        if (a.do_outputs) {
-            const int64_t poff = (int64_t)f * a.plane_stride;
-            const int64_t soff = (int64_t)f * a.slot_stride;
-            if (!board) column_pass(g, s, t);  // else copied with the board
-            fog_pass(g, s, alive, t);  // counts the land
-            if constexpr (MULTI) {
-                if (t.lane < g.P) {
-                    a.scoreboard[2 * (soff + g.player_off + t.lane) + 0] = s.misc[8 + t.lane];
-                    a.scoreboard[2 * (soff + g.player_off + t.lane) + 1] = s.misc[16 + t.lane];
-                }
-            }
-            if (a.next_actions)
-                output_pass<true, true, LW>(a, g, s, alive, fin, t, poff);
-            else
-                output_pass<true, false, LW>(a, g, s, alive, fin, t, poff);
-            if constexpr (!MULTI) {
-                if (t.lane < g.P) {
-                    a.reward[soff + g.player_off + t.lane] = my_reward;
-                    a.scoreboard[2 * (soff + g.player_off + t.lane) + 0] = s.misc[8 + t.lane];
-                    a.scoreboard[2 * (soff + g.player_off + t.lane) + 1] = s.misc[16 + t.lane];
-                }
-                if (t.lane == 0) a.done[(int64_t)f * a.game_stride + gidx] = (uint8_t)done;
-            }
-        } else if (a.next_actions) {
-            output_pass<false, true, LW>(a, g, s, alive, fin, t, 0);
-        }
-        if (a.next_actions) my_act = policy_pass<!MULTI, LW>(a, g, s, alive, fin, frame, game_id_of<UNI>(a, gidx), t);
+        finish_frame<MULTI, LW, UNI>(a, g, s, gidx, f, true, alive, finished != 0, frame, my_reward, done, my_act, t);
     }
     if (MULTI && a.next_actions && t.lane < g.P) a.next_actions[g.player_off + t.lane] = my_act;
     if (wrote_state) {
         t.sync();
         store_board(a, g, s, t);
     }
-    if (t.lane == 0 && a.op != OP_OBSERVE && a.op != OP_POLICY) {
-        uint4* dst = reinterpret_cast<uint4*>(sc);
-        dst[0] = make_uint4(turn, frame, epoch, alive);
-        dst[1] = make_uint4(finished, invalid, saturated, a.op == OP_CREATE ? 0u : err);
-    }
+    if (t.lane == 0 && a.op != OP_OBSERVE && a.op != OP_POLICY)
+        store_scalars(a, gidx, turn, frame, epoch, alive, finished, invalid, saturated, err);
 }
 
 
@@ -1441,9 +1446,8 @@ __device__ __forceinline__ void run_game(const KArgs& a, const Smem& s, char* wa
 
 // One game per group of LW lanes (32: a warp; 16 or 8: two or four games per
 // warp); groups walk the item list with a grid stride.  MULTI: several frames
-// per launch (rollouts) with the board kept in shared memory.  SPAWN: the map
-// generator with spawn options (LW = 32 only).  UNI: every game of the launch
-// has the launch's shape (uniform batches).
+// per launch (rollouts) with the board kept in shared memory.  UNI: every
+// game of the launch has the launch's shape (uniform batches).
 // Register budget: 64 per thread (4 CTAs of 8 warps per SM) for the per-frame
 // form; the multi-frame form keeps more state live across frames and runs
 // best with 85 (3 CTAs).
@@ -1480,7 +1484,7 @@ __global__ void __launch_bounds__(256, MULTI ? 3 : 4) k_generals(const KArgs a) 
 // runs one game per lane group: two per warp for two-player buckets of small
 // boards, one per warp otherwise.  The CTA waits at a barrier between items,
 // so that the next item may carve the same bytes differently.
-template <bool MULTI>
+template <bool MULTI, bool SPAWN>
 __global__ void __launch_bounds__(256, MULTI ? 3 : 4) k_worklist(const KArgs a, const WArgs w) {
     chain_entry();
     extern __shared__ __align__(16) char smem_raw[];
@@ -1511,14 +1515,14 @@ __global__ void __launch_bounds__(256, MULTI ? 3 : 4) k_worklist(const KArgs a, 
             const int grp = 2 * warp + (wl >> 4);
             if (grp < item.count) {
                 char* base = smem_raw + grp * bg.group_smem;
-                run_game<MULTI, false, 16, false>(a, carve_geom(base, bg.geom), base, bg.geom,
+                run_game<MULTI, SPAWN, 16, false>(a, carve_geom(base, bg.geom), base, bg.geom,
                                                   w.order[item.first + grp], t);
             }
         } else {
             const Grp<32> t(wl);
             if (warp < item.count) {
                 char* base = smem_raw + warp * bg.group_smem;
-                run_game<MULTI, false, 32, false>(a, carve_geom(base, bg.geom), base, bg.geom,
+                run_game<MULTI, SPAWN, 32, false>(a, carve_geom(base, bg.geom), base, bg.geom,
                                                   w.order[item.first + warp], t);
             }
         }
@@ -1546,20 +1550,53 @@ __global__ void k_copy(const uint4* __restrict__ src, uint4* __restrict__ dst, s
     for (; i < n; i += stride) __stcs(dst + i, __ldcs(src + i));
 }
 
+using StepKernel = void (*)(KArgs);
+using WorklistKernel = void (*)(KArgs, WArgs);
+
+// The step kernel of a launch: lw lanes per game (8 only in multi-frame
+// launches of the plain generator).  The spawn options have kernels of their
+// own, since the generator with them sets the registers of a kernel that
+// only calls it (compiled into the plain ones: 324 -> 359 us for 64 frames of
+// 1,024 games, 240 -> 251 us per frame of the mixed batch's work list).
+StepKernel step_kernel(int lw, bool multi, bool uniform, bool spawn) {
+    if (!multi && spawn) {
+        if (lw == 32) return k_generals<false, true, 32, false>;
+        return uniform ? k_generals<false, true, 16, true> : k_generals<false, true, 16, false>;
+    }
+    if (!multi) {
+        if (lw == 32) return uniform ? k_generals<false, false, 32, true> : k_generals<false, false, 32, false>;
+        return uniform ? k_generals<false, false, 16, true> : k_generals<false, false, 16, false>;
+    }
+    if (spawn) return lw == 32 ? k_generals<true, true, 32, false> : k_generals<true, true, 16, false>;
+    if (lw == 32) return uniform ? k_generals<true, false, 32, true> : k_generals<true, false, 32, false>;
+    if (lw == 16) return uniform ? k_generals<true, false, 16, true> : k_generals<true, false, 16, false>;
+    return uniform ? k_generals<true, false, 8, true> : k_generals<true, false, 8, false>;
+}
+WorklistKernel worklist_kernel(bool multi, bool spawn) {
+    if (!multi) return spawn ? k_worklist<false, true> : k_worklist<false, false>;
+    return spawn ? k_worklist<true, true> : k_worklist<true, false>;
+}
+
+bool has_spawn_options(const KArgs& a) { return a.spawn_dmax > 0 || a.spawn_bfs || a.castle_radius > 0; }
+
 // Every step-kernel instantiation may take up to the per-CTA maximum of
 // dynamic shared memory on the current device: set once per device, so no
 // launch shape needs its own opt-in (the limit gates launches only).
 int allow_max_smem() {
     static SmemLimit limit;
-    const void* fns[14] = {
-        (const void*)k_generals<false, false, 32, false>, (const void*)k_generals<true, false, 32, false>,
-        (const void*)k_generals<false, false, 32, true>,  (const void*)k_generals<true, false, 32, true>,
-        (const void*)k_generals<false, false, 16, false>, (const void*)k_generals<true, false, 16, false>,
-        (const void*)k_generals<false, false, 16, true>,  (const void*)k_generals<true, false, 16, true>,
-        (const void*)k_generals<false, false, 8, false>,  (const void*)k_generals<true, false, 8, false>,
-        (const void*)k_generals<false, false, 8, true>,   (const void*)k_generals<true, false, 8, true>,
-        (const void*)k_generals<false, true, 32, false>,  (const void*)k_generals<true, true, 32, false>};
-    return limit.raise(fns, 14, 227 * 1024);
+    static const void* fns[15];
+    static std::once_flag once;
+    std::call_once(once, [] {
+        int n = 0;
+        for (int uniform = 0; uniform < 2; ++uniform) {
+            for (int lw : {32, 16}) fns[n++] = (const void*)step_kernel(lw, false, uniform, false);
+            for (int lw : {32, 16, 8}) fns[n++] = (const void*)step_kernel(lw, true, uniform, false);
+        }
+        for (int multi = 0; multi < 2; ++multi)
+            for (int lw : {32, 16}) fns[n++] = (const void*)step_kernel(lw, multi, false, true);
+        fns[n++] = (const void*)step_kernel(16, false, true, true);
+    });
+    return limit.raise(fns, 15, 227 * 1024);
 }
 
 uint32_t bucket_geom(int npad_max, int nw_stride, int pmax, bool narrow) {
@@ -1570,7 +1607,8 @@ int worklist_shape(bool multi, int* cta_smem, int* ctas) {
     // four CTAs of 8 warps per SM per frame (the register budget's limit),
     // three in multi-frame launches; each takes an equal share of the SM's
     // shared memory less the per-CTA reservation
-    const void* f = multi ? (const void*)k_worklist<true> : (const void*)k_worklist<false>;
+    // (the same shape with spawn options: their kernel has the same budget)
+    const void* f = (const void*)worklist_kernel(multi, false);
     int dev = 0, sms = 0, smem_sm = 0, reserved = 0;
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return (int)e;
@@ -1582,6 +1620,9 @@ int worklist_shape(bool multi, int* cta_smem, int* ctas) {
     if (bytes > 227 * 1024) bytes = 227 * 1024;
     // the kernel's own static slot counts against the per-CTA limit too
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess)
+        return (int)e;
+    if ((e = cudaFuncSetAttribute((const void*)worklist_kernel(multi, true), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  bytes)) != cudaSuccess)
         return (int)e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 256, (size_t)bytes)) != cudaSuccess)
@@ -1597,8 +1638,7 @@ int launch_worklist(const KArgs& a, const WArgs& w, int cta_smem, int ctas, void
     const bool multi = a.frames > 1 || a.action_log;
     const int grid = ctas < w.n_items ? ctas : w.n_items;
     if (grid <= 0) return 0;
-    if (multi) return launch_chained(k_worklist<true>, dim3(grid), dim3(256), cta_smem, st, a, w);
-    return launch_chained(k_worklist<false>, dim3(grid), dim3(256), cta_smem, st, a, w);
+    return launch_chained(worklist_kernel(multi, has_spawn_options(a)), dim3(grid), dim3(256), cta_smem, st, a, w);
 }
 
 int warp_smem_bytes(int npad_max, int pmax, int* nw_stride, bool narrow) {
@@ -1683,37 +1723,22 @@ int pick_warps(const void* f, int fixed, int games_per_warp, int warp_smem, int 
     return w;
 }
 
-// The plain-generator kernels of one lane-group width: per frame or
-// multi-frame, for uniform or per-game shapes.
-template <int LW>
-const void* plain_kernel(bool multi, bool uniform) {
-    if (multi && uniform) return (const void*)k_generals<true, false, LW, true>;
-    if (multi) return (const void*)k_generals<true, false, LW, false>;
-    if (uniform) return (const void*)k_generals<false, false, LW, true>;
-    return (const void*)k_generals<false, false, LW, false>;
-}
-
-template <int LW>
-int launch_plain(const KArgs& a, bool multi, int fixed_warps, int max_ctas, int sms, cudaStream_t st) {
-    constexpr int kPerWarp = 32 / LW;
-    const void* f = plain_kernel<LW>(multi, a.uniform != 0);
-    const int warps = pick_warps(f, fixed_warps, kPerWarp, a.warp_smem, a.n_items, sms);
-    const int games_per_cta = kPerWarp * warps;
+int launch_groups(const KArgs& a, int lw, bool multi, bool spawn, int fixed_warps, int max_ctas, int sms,
+                  cudaStream_t st) {
+    const StepKernel f = step_kernel(lw, multi, a.uniform != 0, spawn);
+    const int per_warp = 32 / lw;
+    const int warps = pick_warps((const void*)f, fixed_warps, per_warp, a.warp_smem, a.n_items, sms);
+    const int games_per_cta = per_warp * warps;
     const int smem = a.warp_smem * games_per_cta;
     int blocks = (a.n_items + games_per_cta - 1) / games_per_cta;
     // multi-frame launches: a grid of many waves, groups stride over any items beyond it
     if (multi && max_ctas > 0 && blocks > 64 * max_ctas) blocks = 64 * max_ctas;
-    const dim3 grid(blocks), block(32 * warps);
-    if (multi && a.uniform) return launch_chained(k_generals<true, false, LW, true>, grid, block, smem, st, a);
-    if (multi) return launch_chained(k_generals<true, false, LW, false>, grid, block, smem, st, a);
-    if (a.uniform) return launch_chained(k_generals<false, false, LW, true>, grid, block, smem, st, a);
-    return launch_chained(k_generals<false, false, LW, false>, grid, block, smem, st, a);
+    return launch_chained(f, dim3(blocks), dim3(32 * warps), smem, st, a);
 }
 
 int launch_step(const KArgs& a, int warps_per_cta, int max_ctas, void* stream) {
     if (a.n_items <= 0) return 0;
 
-    const bool spawn = a.spawn_dmax > 0 || a.spawn_bfs || a.castle_radius > 0;
     const bool multi = a.frames > 1 || a.action_log;
     const cudaStream_t st = (cudaStream_t)stream;
     {
@@ -1729,37 +1754,25 @@ int launch_step(const KArgs& a, int warps_per_cta, int max_ctas, void* stream) {
         sms = n > 0 ? n : 1;
         sm_count.store(sms, std::memory_order_relaxed);
     }
-    // several games per warp for small two-player boards, plain generator
-    // only, once the batch is large enough: below it a warp per game is
+    // several games per warp for small two-player boards, once the batch is large enough: below it a warp per game is
     // faster (measured on 24x24 1v1: 1,024 games per frame 98 against 87 M
     // frames/s, resident 194 against 122 M; pairs win from 2,048 games per
     // frame and 4,096 resident)
     const bool large = a.n_items >= (multi ? 24 : 12) * sms;
-    const bool small = !spawn && a.pmax <= kPairMaxPlayers && (a.lane_groups == 2 || (a.lane_groups == 0 && large));
+    const bool small = a.pmax <= kPairMaxPlayers && (a.lane_groups == 2 || (a.lane_groups == 0 && large));
     const int wcap = warps_per_cta > 0 ? warps_per_cta : 1;  // the fixed shape must fit too
     // narrow groups keep their legal moves as chunk masks: a larger carve
     const int ws_narrow = small ? warp_smem_bytes(a.npad_max, a.pmax, nullptr, true) : a.warp_smem;
     int per_warp = 1;
-    if (small && multi && a.npad_max <= kQuadMaxCells && 4 * wcap * ws_narrow <= 227 * 1024)
+    const bool spawn = has_spawn_options(a);
+    if (small && multi && !spawn && a.npad_max <= kQuadMaxCells && 4 * wcap * ws_narrow <= 227 * 1024)
         per_warp = 4;
     else if (small && a.npad_max <= kPairMaxCells && 2 * wcap * ws_narrow <= 227 * 1024)
         per_warp = 2;
-    if (per_warp > 1) {
-        KArgs n = a;
-        n.warp_smem = ws_narrow;
-        return per_warp == 4 ? launch_plain<8>(n, multi, warps_per_cta, max_ctas, sms, st)
-                             : launch_plain<16>(n, multi, warps_per_cta, max_ctas, sms, st);
-    }
-    if (spawn) {  // one game per warp, shapes read per game
-        const void* f = multi ? (const void*)k_generals<true, true, 32, false> : (const void*)k_generals<false, true, 32, false>;
-        const int warps = pick_warps(f, warps_per_cta, 1, a.warp_smem, a.n_items, sms);
-        const int smem = a.warp_smem * warps;
-        int blocks = (a.n_items + warps - 1) / warps;
-        if (multi && max_ctas > 0 && blocks > 64 * max_ctas) blocks = 64 * max_ctas;
-        if (multi) return launch_chained(k_generals<true, true, 32, false>, dim3(blocks), dim3(32 * warps), smem, st, a);
-        return launch_chained(k_generals<false, true, 32, false>, dim3(blocks), dim3(32 * warps), smem, st, a);
-    }
-    return launch_plain<32>(a, multi, warps_per_cta, max_ctas, sms, st);
+    if (per_warp == 1) return launch_groups(a, 32, multi, spawn, warps_per_cta, max_ctas, sms, st);
+    KArgs n = a;
+    n.warp_smem = ws_narrow;
+    return launch_groups(n, 32 / per_warp, multi, spawn, warps_per_cta, max_ctas, sms, st);
 }
 
 int launch_copy(const void* src, void* dst, size_t n16, int blocks, void* stream) {

@@ -285,6 +285,18 @@ def test_generator_options_match_oracle(opts):
     rollout_policy(env, orc, 70, policy_seed=5, check_every=2, tag=str(opts))
 
 
+@pytest.mark.parametrize("lanes", [1, 2])
+@pytest.mark.parametrize("H,W,mode,P", [(32, 32, 0, 2), (31, 33, 0, 2), (33, 31, 2, 3), (16, 64, 0, 2), (64, 16, 0, 2),
+                                        (1, 40, 0, 2), (40, 1, 1, 4), (32, 31, 2, 8)])
+def test_generator_rows_at_word_edges(H, W, mode, P, lanes):
+    """The generator's row bitsets where a row fills its word, takes a wider
+    one or the group's lanes hold several rows, with every option, through resets."""
+    full = lambda x: np.full(24, x, np.int32)  # noqa: E731
+    env, orc = pair(full(H), full(W), full(mode), full(P), lanes=lanes, seed=23, n_cities=5, max_turns=7,
+                    bfs_distance=1, min_general_dist=9, castle_radius=4)
+    rollout_policy(env, orc, 16, policy_seed=3, check_every=1, tag=f"{H}x{W}")
+
+
 def test_spawn_range_curriculum_update():
     import torch
     G = 48
