@@ -298,7 +298,6 @@ int gen_set_launch(gen_env *env, int warps_per_cta);
  *  - games per warp (gen_set_lane_groups: by batch size, one, or several);
  *  - for batches of several size buckets, the batch form (gen_set_batch_form);
  *  - the rollout form that GEN_ROLLOUT_AUTO runs (8-frame rollouts, per frame);
- *  - the sampler form (gen_set_sample_form, on zero logits);
  *  - each size bucket's games per CTA among 2, 4, 8 in the bucket form.
  * Results are cached for the process per batch signature (bucket classes
  * and counts, SM count).  `steps` timed calls per candidate; a
@@ -460,13 +459,10 @@ int gen_set_lane_groups(gen_env *env, int mode);
  * GEN_ERR_BAD_ARG for NULL env or a form outside 0..2. */
 int gen_set_batch_form(gen_env *env, int form);
 
-/* Tuning call, no counterpart in the paper.  How gen_sample_actions
- * spreads a game over the GPU (the results are the same): 1 = one warp per
- * game, players in turn; 2 = one CTA per game with a warp per player (as
- * many as fit in shared memory beside the board); 3 = one CTA per player
- * with a thread per (own cell, entry) pair; 0 (default) = 3 while games x
- * the most players per game is at most 8 x the SM count, else 2.
- * GEN_ERR_BAD_ARG for NULL env or a form outside 0..3. */
+/* Tuning call, no counterpart in the paper; kept for its callers.  It chose
+ * between ways to spread gen_sample_actions over the GPU; a warp per player
+ * is now the fastest at every batch size and always runs, so the form (0..3)
+ * changes nothing.  GEN_ERR_BAD_ARG for NULL env or a form outside 0..3. */
 int gen_set_sample_form(gen_env *env, int form);
 
 /* ---- feature tensor (App. A, table of observation channels) -------------

@@ -77,7 +77,6 @@ struct gen_env {
     int player_slots = 0;
     int pmax = 0;
     int npad_max = 0;
-    int sample_form = 0;  // gen_sample_actions: 1 a warp per game, 2 a CTA per game, 3 a CTA per player, 0 by batch size
     int rollout_form = GEN_ROLLOUT_RESIDENT;  // what GEN_ROLLOUT_AUTO runs (the autotuner's pick)
     int lane_groups = 0;  // step kernels: 0 by batch size, 1 a warp per game, 2 several per warp when allowed
     int nmax = 0;
@@ -1423,7 +1422,12 @@ int gen_sample_actions(gen_env* e, const float* d_logits, uint64_t seed, int32_t
     a.actions = d_actions;
     a.mask9 = d_mask9;
     a.npad_max = e->npad_max;
-    const int rc = gk::launch_sample(a, e->pmax, e->sample_form, stream);
+    if (e->uniform) {
+        a.uniform = 1;
+        a.ushape = e->h_info[0];
+        a.game_id_base = e->prm.game_id_base;
+    }
+    const int rc = gk::launch_sample(a, e->pmax, stream);
     if (rc != 0) return cuda_fail((cudaError_t)rc, "sampler launch");
     return GEN_OK;
 }
@@ -1447,7 +1451,6 @@ int gen_set_batch_form(gen_env* e, int form) {
 int gen_set_sample_form(gen_env* e, int form) {
     if (!e) return fail(GEN_ERR_BAD_ARG, "env is NULL");
     if (form < 0 || form > 3) return fail(GEN_ERR_BAD_ARG, "form %d outside [0, 3]", form);
-    e->sample_form = form;
     return GEN_OK;
 }
 
@@ -1473,7 +1476,7 @@ int gen_set_launch(gen_env* e, int warps_per_cta) {
 
 // The environment-wide launch choices of the autotuner, per batch signature.
 struct TunedForms {
-    int lane_groups, batch_form, rollout_form, sample_form;
+    int lane_groups, batch_form, rollout_form;
 };
 static std::map<std::string, TunedForms> g_forms_cache;  // under g_tune_mu
 
@@ -1494,9 +1497,8 @@ static int tune_env_forms(gen_env* e, int steps, int sms, std::string& rep) {
             e->lane_groups = f.lane_groups;
             e->batch_form = f.batch_form;
             e->rollout_form = f.rollout_form;
-            e->sample_form = f.sample_form;
-            snprintf(line, sizeof(line), "forms (cached): lanes %d, batch %d, rollout %d, sampler %d\n", f.lane_groups,
-                     f.batch_form, f.rollout_form, f.sample_form);
+            snprintf(line, sizeof(line), "forms (cached): lanes %d, batch %d, rollout %d\n", f.lane_groups,
+                     f.batch_form, f.rollout_form);
             rep += line;
             return build_worklist(e);
         }
@@ -1513,7 +1515,6 @@ static int tune_env_forms(gen_env* e, int steps, int sms, std::string& rep) {
     if (rc) return rc;
     constexpr int K = 8;
     gen_outputs ko{};
-    float* logits = nullptr;
     cudaStream_t s = nullptr;
     cudaEvent_t a = nullptr, b = nullptr;
     const size_t pc = (size_t)t->plane_cells, ps = (size_t)t->player_slots, G = (size_t)t->G;
@@ -1528,12 +1529,10 @@ static int tune_env_forms(gen_env* e, int steps, int sms, std::string& rep) {
     if (ce == cudaSuccess) ce = cudaMalloc(&ko.reward, K * ps * 4);
     if (ce == cudaSuccess) ce = cudaMalloc(&ko.scoreboard, K * ps * 8);
     if (ce == cudaSuccess) ce = cudaMalloc(&ko.done, K * G);
-    if (ce == cudaSuccess) ce = cudaMalloc(&logits, pc * 9 * sizeof(float));
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(logits, 0, pc * 9 * sizeof(float), s);
     if (ce != cudaSuccess) rc = cuda_fail(ce, "autotune scratch");
     if (rc == GEN_OK) rc = ensure_internal_outputs(t);
     if (rc == GEN_OK) rc = gen_policy(t, 1, t->d_actions, s);
-    TunedForms best{e->lane_groups, e->batch_form, e->rollout_form, e->sample_form};
+    TunedForms best{e->lane_groups, e->batch_form, e->rollout_form};
     auto step = [&]() { return gen_step_policy(t, t->d_actions, &t->d_out, 1, t->d_actions, s); };
     if (rc == GEN_OK) {
         // lane groups: by batch size, a warp per game, or several per warp where the games allow
@@ -1583,22 +1582,7 @@ static int tune_env_forms(gen_env* e, int steps, int sms, std::string& rep) {
         }
         rep += "\n";
     }
-    if (rc == GEN_OK) {
-        float bt = 1e30f;
-        rep += "sampler:";
-        for (int form : {1, 2, 3}) {
-            t->sample_form = form;
-            auto samp = [&]() { return gen_sample_actions(t, logits, 1, t->d_actions, nullptr, s); };
-            const float ms = time_calls(samp, steps, s, a, b);
-            snprintf(line, sizeof(line), " %d=%.4fms", form, ms);
-            rep += line;
-            if (ms < bt) {
-                bt = ms;
-                best.sample_form = form;
-            }
-        }
-        rep += "\n";
-    }
+    rep += "sampler: a warp per player at every batch size\n";
     cudaFree(ko.obs_army);
     cudaFree(ko.obs_owner);
     cudaFree(ko.obs_terrain);
@@ -1607,7 +1591,6 @@ static int tune_env_forms(gen_env* e, int steps, int sms, std::string& rep) {
     cudaFree(ko.reward);
     cudaFree(ko.scoreboard);
     cudaFree(ko.done);
-    cudaFree(logits);
     if (a) cudaEventDestroy(a);
     if (b) cudaEventDestroy(b);
     if (s) cudaStreamDestroy(s);
@@ -1616,7 +1599,6 @@ static int tune_env_forms(gen_env* e, int steps, int sms, std::string& rep) {
     e->lane_groups = best.lane_groups;
     e->batch_form = best.batch_form;
     e->rollout_form = best.rollout_form;
-    e->sample_form = best.sample_form;
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         g_forms_cache[sig] = best;

@@ -173,7 +173,7 @@ struct FArgs {
 // any game.  Returns a cudaError_t.
 int launch_features(const FArgs& f, int pmax, int form, void* stream);
 
-// Policy sampling over the H x W x 9 action space: one warp per game.
+// Policy sampling over the H x W x 9 action space.
 struct SArgs {
     const GameInfo* info;
     const int16_t* army;
@@ -186,12 +186,16 @@ struct SArgs {
     int32_t* actions;       // [player slots] (NULL with logits NULL)
     uint8_t* mask9;         // optional: 9 * Npad legal-entry bytes per player plane at q * 9
     int32_t npad_max;       // largest board (cells, multiple of 16)
+    // uniform batch: as in KArgs
+    int32_t uniform;
+    GameInfo ushape;
+    uint64_t game_id_base;
 };
 
-// Launch the sampler over every game on `stream`: form 1 one warp per game,
-// 2 (and 0, the default) one CTA per game with a warp per player.  pmax = the most
+// Launch the sampler (and the expanded mask, when mask9 is given; only the
+// mask when logits is NULL) over every game on `stream`.  pmax = the most
 // players of any game.  Returns a cudaError_t.
-int launch_sample(const SArgs& a, int pmax, int form, void* stream);
+int launch_sample(const SArgs& a, int pmax, void* stream);
 
 // Bytes of shared memory one lane group needs for games up to npad_max
 // cells and pmax players; also returns the bitset stride in words.  narrow:

@@ -17,27 +17,11 @@
 // single-precision operation with round-to-nearest written out explicitly
 // (no contraction), so the weights are bit-reproducible.
 //
-// One CTA per game with a warp per player (k_sample_cta), one warp per game
-// with the players in turn (k_sample), or, for small batches, one CTA per
-// player with a thread per (own cell, entry) pair (k_sample_wide, described
-// where it is defined).  The board is staged in
-// shared memory (every 16-byte copy in flight at once); legal entries lie
-// only on the player's own cells, so the warp first lists those cells in
-// index order (a ballot per 32 cells, no global load) and the passes run over
-// the list, 32 own cells at a time: pass 1 derives each cell's nine legal
-// bits and takes the maximum; pass 2 (logits held in registers for the first
-// 64 own cells, read again from L1/L2 beyond) sums each cell's weights,
-// computing every exponential once (two entries per packed FMA chain), and
-// keeps the sums per cell and per 32
-// cells; pass 3 finds the group, the cell and (nine lanes weighing the cell's
-// entries at once) the entry where the running sum first exceeds r.  Only the
-// own cells' logits are read (36 bytes each).  The expanded mask, when asked
-// for, is a dense pass over every cell (a cell's entries belong to its owner)
-// written through shared memory with 16-byte stores.
+// One warp per player (k_sample_slots), the expanded mask a CTA per game
+// (k_mask9), both at once in one launch (k_sample_mask).
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cstdint>
 
 #include "gk_internal.h"
@@ -46,8 +30,9 @@ namespace gk {
 namespace {
 
 constexpr unsigned kAll = 0xFFFFFFFFu;
-constexpr int kWarps = 8;
 constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
+constexpr float kNegInf = -__builtin_huge_valf();
+constexpr float kLowest = -3.402823466e38f;
 
 __device__ __forceinline__ uint64_t mix64(uint64_t z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -80,9 +65,11 @@ __device__ __forceinline__ uint32_t weight_shift(float l, float m) {
     return n >= 0 ? sig << 1 : sig >> (-(n + 1));
 }
 
-// two weights at once: the same single-precision operations as
-// weight_shift, issued as packed pairs (each half an IEEE round-to-nearest
-// operation of its own, so the results are bit for bit those of two calls)
+// Two weights at once: the same single-precision operations as weight_shift,
+// issued as packed pairs (each half an IEEE operation of its own), for finite
+// m >= l (l = -inf included: weight 0).  floor(t) is the round-down sum with
+// 1.5 * 2^23, whose low bits are the integer (no conversion instruction), and
+// the shift 24-bit significand << 1 >> -n is 0 from n = -26 on by itself.
 __device__ __forceinline__ uint64_t pack2(float a, float b) {
     return (uint64_t)__float_as_uint(a) | ((uint64_t)__float_as_uint(b) << 32);
 }
@@ -93,26 +80,59 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
-__device__ __forceinline__ uint32_t weight_from(float t, float nf, float p) {
-    if (t < -25.0f) return 0u;
-    const int n = (int)nf;
-    const uint32_t sig = (__float_as_uint(p) & 0x7FFFFFu) | 0x800000u;
-    return n >= 0 ? sig << 1 : sig >> (-(n + 1));
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
-__device__ __forceinline__ uint2 weight_shift2(float l0, float l1, float m) {
-    const float t0 = __fmul_rn(__fsub_rn(l0, m), 1.4426950408889634f);
-    const float t1 = __fmul_rn(__fsub_rn(l1, m), 1.4426950408889634f);
-    const float n0 = floorf(t0), n1 = floorf(t1);
-    const uint64_t f = pack2(__fsub_rn(t0, n0), __fsub_rn(t1, n1));
-    uint64_t p = pack2(1.5252733804059838e-05f, 1.5252733804059838e-05f);
-    p = fma2(p, f, pack2(0.00015403530393381606f, 0.00015403530393381606f));
-    p = fma2(p, f, pack2(0.0013333558146428441f, 0.0013333558146428441f));
-    p = fma2(p, f, pack2(0.009618129107628477f, 0.009618129107628477f));
-    p = fma2(p, f, pack2(0.055504108664821576f, 0.055504108664821576f));
-    p = fma2(p, f, pack2(0.2402265069591007f, 0.2402265069591007f));
-    p = fma2(p, f, pack2(0.6931471805599453f, 0.6931471805599453f));
-    p = fma2(p, f, pack2(1.0f, 1.0f));
-    return make_uint2(weight_from(t0, n0, lo2(p)), weight_from(t1, n1, hi2(p)));
+__device__ __forceinline__ uint64_t add2_down(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t both(float x) { return pack2(x, x); }
+constexpr float kFloorMagic = 12582912.0f;  // 1.5 * 2^23, bits 0x4B400000
+__device__ __forceinline__ uint32_t weight_bits(float p, float r) {
+    // P in [1, 2) (at most 1.9999988, at f = 1): its significand << 1 from the bits 0x3F800000 + mantissa
+    const uint32_t sig = 2u * __float_as_uint(p) + 0x82000000u;
+    return __funnelshift_rc(sig, 0u, 0x4B400000u - __float_as_uint(r));
+}
+// sum of the weights of l0 and l1
+__device__ __forceinline__ uint32_t weight_pair(float l0, float l1, uint64_t minus_m) {
+    uint64_t t = mul2(add2(pack2(l0, l1), minus_m), both(1.4426950408889634f));
+    t = pack2(fmaxf(lo2(t), -64.0f), fmaxf(hi2(t), -64.0f));
+    const uint64_t r = add2_down(t, both(kFloorMagic));
+    const uint64_t f = add2(t, fma2(r, both(-1.0f), both(kFloorMagic)));
+    uint64_t p = both(1.5252733804059838e-05f);
+    p = fma2(p, f, both(0.00015403530393381606f));
+    p = fma2(p, f, both(0.0013333558146428441f));
+    p = fma2(p, f, both(0.009618129107628477f));
+    p = fma2(p, f, both(0.055504108664821576f));
+    p = fma2(p, f, both(0.2402265069591007f));
+    p = fma2(p, f, both(0.6931471805599453f));
+    p = fma2(p, f, both(1.0f));
+    return weight_bits(lo2(p), lo2(r)) + weight_bits(hi2(p), hi2(r));
+}
+// sum of the weights of one cell's nine entries (-inf: illegal)
+__device__ __forceinline__ uint32_t cell_weight(const float (&v)[9], float m) {
+    const uint64_t mm = both(-m);
+    uint32_t w = 0u;
+#pragma unroll
+    for (int k = 0; k < 8; k += 2) w += weight_pair(v[k], v[k + 1], mm);
+    return w + weight_pair(v[8], kNegInf, mm);
+}
+// of two cells
+__device__ __forceinline__ uint32_t cell_weight2(const float (&v)[9], const float (&u)[9], float m) {
+    const uint64_t mm = both(-m);
+    uint32_t w = 0u;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) w += weight_pair(v[k], u[k], mm);
+    return w;
 }
 
 // legal entries of one cell for player p as bits 0..8 (entry k of the cell)
@@ -126,29 +146,18 @@ __device__ __forceinline__ uint32_t legal9(int own_p, int army, uint32_t terrain
     return b;
 }
 
-// shared memory of one warp's player, sized for boards up to npad_max cells:
-// the player's own cells in index order (2 B), their legal bits (2 B) and
-// weight sums (4 B), the weight sum of every 32 of them (8 B), mask staging
-// (288 B); a multiple of 16 bytes.  The board (4 B per cell) comes first.
-__host__ __device__ __forceinline__ int sample_player_bytes(int npad_max) {
-    const int rounds = (npad_max + 31) >> 5;
-    return 8 * npad_max + 8 * ((rounds + 1) & ~1) + 288;
-}
-__host__ __device__ __forceinline__ int sample_warp_bytes(int npad_max) {
-    return 4 * npad_max + sample_player_bytes(npad_max);
-}
-
-// the nine logits of one cell, every load issued before any is used
-__device__ __forceinline__ void load9(float (&v)[9], const float* x) {
-#pragma unroll
-    for (int k = 0; k < 9; ++k) v[k] = __ldcg(x + k);
+// a game's description; of a uniform batch without a load, since the loads
+// that follow would wait for it
+__device__ __forceinline__ GameInfo sample_game(const SArgs& a, int gidx) {
+    if (!a.uniform) return a.info[gidx];
+    GameInfo gi = a.ushape;
+    gi.cell_off = gidx * gi.Npad;
+    gi.player_off = gidx * gi.P;
+    gi.plane_off = (int64_t)gidx * gi.P * gi.Npad;
+    gi.game_id = a.game_id_base + (uint64_t)gidx;
+    return gi;
 }
 
-__device__ __forceinline__ uint64_t warp_sum64(uint64_t x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kAll, x, o);
-    return x;
-}
 __device__ __forceinline__ uint64_t warp_incl64(uint64_t x, int lane) {
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -158,474 +167,280 @@ __device__ __forceinline__ uint64_t warp_incl64(uint64_t x, int lane) {
     return x;
 }
 
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
-                 "l"(gmem)
-                 : "memory");
-}
+// ---- a warp per player ------------------------------------------------------
+// The player's own cells are listed in index order (2 B each in shared
+// memory): a lane compares 32 owner bytes, one scan places them all on boards
+// of up to 1,024 cells.  Lane l then takes the cells k*l .. k*l + k-1 of the
+// list, k = ceil(cells / 32), so that one 64-bit scan of the lanes' weight
+// sums gives both S and the lane where the running sum first exceeds r; the
+// entry is found with a lane per (cell, entry) of that lane's cells.
+// Nothing is staged: armies and terrain are gathered for the own cells only,
+// in flight with their logits.  A cell's nine logits start at any multiple of
+// 4 bytes, and the three 16-byte vectors around them always hold all nine.
+//
+// Bound by instructions and L1 wavefronts (65,536 1v1 games of 24x24 at mid-
+// game, N(0, 2) logits; the sectors of the own cells' logits and the board
+// need 79 us): 270 -> 143.6 us, 1,531 -> 952 warp instructions per player,
+// against a warp per player that staged the board, loaded each logit by
+// itself and summed and scanned every 32 cells; 1,000 such games 7.9 -> 7.4,
+// 8,192 mixed games of 20..40 a side 243 -> 51 us (shared memory for eight
+// staged players held those to four warps per scheduler).  The other spreads
+// were slower at every size measured, 1 to 65,536 games and 15 to 177 own
+// cells: 512 games 4.2 us against 6.9 us for a warp per game and 5.6 us for a
+// CTA per player with a thread per (cell, entry).
+// 36 warps per SM (56 registers): 148 us where 32 gave 157 us and 40, with
+// spills, 147 us.
+__host__ __device__ __forceinline__ int list_bytes(int npad_max) { return (2 * npad_max + 15) & ~15; }
 
-// a game's board in shared memory, by `nthreads` threads from `tid` on
-__device__ __forceinline__ void stage_board(const SArgs& a, const GameInfo& gi, char* b, int np, int tid, int nthreads) {
-    const uint4* ga = reinterpret_cast<const uint4*>(a.army + gi.cell_off);
-    const uint4* go = reinterpret_cast<const uint4*>(a.owner + gi.cell_off);
-    const uint4* gt = reinterpret_cast<const uint4*>(a.terrain + gi.cell_off);
-    uint4* sa = reinterpret_cast<uint4*>(b);
-    uint4* so = reinterpret_cast<uint4*>(b + 2 * np);
-    uint4* st = reinterpret_cast<uint4*>(b + 3 * np);
-    const int n16 = gi.Npad >> 4;
-    for (int v = tid; v < 2 * n16; v += nthreads) cp_async16(sa + v, ga + v);
-    for (int v = tid; v < n16; v += nthreads) {
-        cp_async16(so + v, go + v);
-        cp_async16(st + v, gt + v);
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-}
-
-// expanded mask rows r0 = row0, row0 + drow, ... (32 cells each) of every
-// player: a cell's legal entries belong to its owner only
-__device__ __forceinline__ void mask_rows(const SArgs& a, const GameInfo& gi, const GameScalars& sc,
-                                          const int16_t* s_army, const int8_t* s_owner, const uint8_t* s_terrain,
-                                          uint8_t* s_mask, int row0, int drow, int lane) {
-    const int N = gi.N, Npad = gi.Npad, P = gi.P;
-    for (int r0 = row0; r0 < Npad; r0 += drow) {
-        const int cells = min(32, Npad - r0), c = r0 + lane;
-        int o = -1;
-        uint32_t lb = 0u;
-        if (c < N) {
-            o = s_owner[c];
-            if (o >= 0) {
-                const bool moves = ((sc.alive >> o) & 1u) && !sc.finished;
-                lb = legal9(true, s_army[c], s_terrain[c], moves);
-            }
-        }
-        const int n16 = (9 * cells) >> 4;
-        for (int p = 0; p < P; ++p) {
-            const uint32_t bits = o == p ? lb : 0u;
-            if (lane < cells)
+// bit j = byte j of the 16 owner bytes O (-1 .. 7) equals p
+__device__ __forceinline__ uint32_t equal_bytes16(uint4 O, uint32_t p4) {
+    const uint32_t o[4] = {O.x, O.y, O.z, O.w};
+    uint32_t z[4];
 #pragma unroll
-                for (int k = 0; k < 9; ++k) s_mask[9 * lane + k] = (uint8_t)((bits >> k) & 1u);
-            __syncwarp();
-            const int64_t base = (gi.plane_off + (int64_t)p * Npad) * 9;
-            if (lane < n16)
-                reinterpret_cast<uint4*>(a.mask9 + base + 9 * r0)[lane] = reinterpret_cast<const uint4*>(s_mask)[lane];
-            __syncwarp();
-        }
-    }
+    for (int q = 0; q < 4; ++q) z[q] = ~(((o[q] ^ p4) & 0x0F0F0F0Fu) + 0x7F7F7F7Fu) & 0x80808080u;  // 0x80 where equal
+    // dot products with powers of two collect the bytes' bits (times 128)
+    const uint32_t lo = __dp4a(z[1], 0x80402010u, __dp4a(z[0], 0x08040201u, 0u));
+    const uint32_t hi = __dp4a(z[3], 0x80402010u, __dp4a(z[2], 0x08040201u, 0u));
+    return (lo >> 7) | (hi << 1);
 }
 
-// player p's action, by one warp over its region `w` of shared memory
+// the nine logits of cell c, -inf where illegal
+__device__ __forceinline__ void load_cell(float (&v)[9], const float* lg, const int16_t* army, const uint8_t* terrain,
+                                          int c, bool moves) {
+    const int s = c & 3;  // the cell's logits start s floats into the vectors
+    const float4* x = reinterpret_cast<const float4*>(lg + (9 * c - s));
+    const float4 a = __ldg(x), b = __ldg(x + 1), d = __ldg(x + 2);
+    const int av = __ldg(army + c);
+    const uint32_t tb = __ldg(terrain + c);
+    const float w[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, d.x, d.y, d.z, d.w};
+    const uint32_t dirs = moves && av >= 2 ? tb >> 2 : 0u;  // neighbour exists and is not a mountain
+    float u[11];
+#pragma unroll
+    for (int k = 0; k < 11; ++k) u[k] = (s & 1) ? w[k + 1] : w[k];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) v[k] = (s & 2) ? u[k + 2] : u[k];
+#pragma unroll
+    for (int d2 = 0; d2 < 4; ++d2) {
+        const bool ok = (dirs >> d2) & 1u;
+        v[1 + d2] = ok ? v[1 + d2] : kNegInf;
+        v[5 + d2] = ok ? v[5 + d2] : kNegInf;
+    }
+}
+// entry e of cell c, -inf where illegal
+__device__ __forceinline__ float legal_logit(const float* lg, const int16_t* army, const uint8_t* terrain, int c, int e,
+                                             bool moves) {
+    const bool ok = e == 0 || (moves && __ldg(army + c) >= 2 && ((uint32_t)__ldg(terrain + c) >> (2 + ((e - 1) & 3))) & 1u);
+    return ok ? __ldg(lg + 9 * c + e) : kNegInf;
+}
+// maximum that is a number only if both are
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float cell_max(const float (&v)[9], float m) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) m = max_nan(m, v[k]);
+    return m;
+}
+__device__ __forceinline__ float warp_max_nan(float m) {
+    asm("redux.sync.max.NaN.f32 %0, %0, 0xffffffff;" : "+f"(m));
+    return m;
+}
+
+// player p's action in game gidx, by one warp; list: its shared memory
 __device__ __forceinline__ int32_t sample_player(const SArgs& a, const GameInfo& gi, const GameScalars& sc, int p,
-                                                 const int16_t* s_army, const int8_t* s_owner,
-                                                 const uint8_t* s_terrain, char* w, int lane) {
-    const int np = a.npad_max, N = gi.N, Npad = gi.Npad;
-    uint32_t* s_w = reinterpret_cast<uint32_t*>(w);                // [np] per own cell
-    uint16_t* s_list = reinterpret_cast<uint16_t*>(w + 4 * np);    // [np] own cells
-    uint16_t* s_legal = reinterpret_cast<uint16_t*>(w + 6 * np);   // [np] per own cell
-    uint64_t* s_round = reinterpret_cast<uint64_t*>(w + 8 * np);   // [rounds]
-    const unsigned lt_mask = (1u << lane) - 1u;
-    const bool moves = ((sc.alive >> p) & 1u) && !sc.finished;
-    const float* lg = a.logits + (gi.plane_off + (int64_t)p * Npad) * 9;
-    // the player's cells in index order (legal entries lie only there)
+                                                 uint16_t* list, int lane) {
+    const uint4* owner = reinterpret_cast<const uint4*>(a.owner + gi.cell_off);
+    const uint32_t p4 = 0x01010101u * (uint32_t)p;
     int n = 0;
-    for (int r0 = 0; r0 < N; r0 += 32) {
-        const int c = r0 + lane;
-        const bool mine = c < N && s_owner[c] == p;
-        const unsigned bal = __ballot_sync(kAll, mine);
-        if (mine) s_list[n + __popc(bal & lt_mask)] = (uint16_t)c;
-        n += __popc(bal);
+    for (int c0 = 0; c0 < gi.Npad; c0 += 1024) {  // 32 cells per lane; padding cells have owner -1
+        const int c = c0 + 32 * lane;
+        const uint4 none = make_uint4(kAll, kAll, kAll, kAll);
+        const uint4 Oa = c < gi.Npad ? __ldg(owner + (c >> 4)) : none;
+        const uint4 Ob = c + 16 < gi.Npad ? __ldg(owner + (c >> 4) + 1) : none;
+        uint32_t mine = equal_bytes16(Oa, p4) | (equal_bytes16(Ob, p4) << 16);
+        const int cnt = __popc(mine);
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kAll, incl, o);
+            if (lane >= o) incl += y;
+        }
+        uint16_t* at = list + n + (incl - cnt);
+        for (; mine; mine &= mine - 1) *at++ = (uint16_t)(c + __ffs(mine) - 1);
+        n += __shfl_sync(kAll, incl, 31);
     }
     __syncwarp();
     if (n == 0) return 0;
-    // pass 1: legal bits and the maximum legal logit; the first two groups'
-    // logits stay in registers for pass 2
-    float m = -3.402823466e38f;
+    const bool moves = ((sc.alive >> p) & 1u) && !sc.finished;
+    const float* lg = a.logits + (gi.plane_off + (int64_t)p * gi.Npad) * 9;
+    const int16_t* army = a.army + gi.cell_off;
+    const uint8_t* terrain = reinterpret_cast<const uint8_t*>(a.terrain + gi.cell_off);
+    const int k = (n + 31) >> 5;
+    const int i0 = lane * k, i1 = min(n, i0 + k);
+    // pass 1: the maximum legal logit; the first two cells stay in registers
     float v0[9], v1[9];
-    for (int i = lane; i < n; i += 32) {
-        const int c = s_list[i];
-        const uint32_t lb = legal9(true, s_army[c], s_terrain[c], moves);
-        s_legal[i] = (uint16_t)lb;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) v0[q] = v1[q] = kNegInf;
+    if (i0 < i1) load_cell(v0, lg, army, terrain, list[i0], moves);
+    if (i0 + 1 < i1) load_cell(v1, lg, army, terrain, list[i0 + 1], moves);
+    float m = cell_max(v1, cell_max(v0, kLowest));
+    for (int i = i0 + 2; i < i1; ++i) {
         float v[9];
-        load9(v, lg + 9 * c);
-#pragma unroll
-        for (int k = 0; k < 9; ++k)
-            if ((lb >> k) & 1u) m = fmaxf(m, v[k]);
-        if (i < 32) {
-#pragma unroll
-            for (int k = 0; k < 9; ++k) v0[k] = v[k];
-        } else if (i < 64) {
-#pragma unroll
-            for (int k = 0; k < 9; ++k) v1[k] = v[k];
-        }
+        load_cell(v, lg, army, terrain, list[i], moves);
+        m = cell_max(v, m);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
-    __syncwarp();
-    // pass 2: weight sums per own cell and per 32 of them (every exponential once)
-    uint64_t S = 0;
-    for (int i0 = 0; i0 < n; i0 += 32) {
-        const int i = i0 + lane;
-        uint32_t wsum = 0u;
-        if (i < n) {
-            const int c = s_list[i];
-            const uint32_t lb = s_legal[i];
+    m = warp_max_nan(m);
+    // pass 2: the lane's weight sum, every exponential once
+    uint64_t mine = 0;
+    if (m < -kNegInf) {
+        mine = k > 1 ? cell_weight2(v0, v1, m) : cell_weight(v0, m);
+        for (int i = i0 + 2; i < i1; ++i) {
             float v[9];
-            if (i0 == 0) {
-#pragma unroll
-                for (int k = 0; k < 9; ++k) v[k] = v0[k];
-            } else if (i0 == 32) {
-#pragma unroll
-                for (int k = 0; k < 9; ++k) v[k] = v1[k];
-            } else {
-                load9(v, lg + 9 * c);
-            }
-#pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-                const uint2 w2 = weight_shift2(v[k], v[k + 1], m);
-                wsum += ((lb >> k) & 1u) ? w2.x : 0u;
-                wsum += ((lb >> (k + 1)) & 1u) ? w2.y : 0u;
-            }
-            if ((lb >> 8) & 1u) wsum += weight_shift(v[8], m);
-            s_w[i] = wsum;
+            load_cell(v, lg, army, terrain, list[i], moves);
+            mine += cell_weight(v, m);
         }
-        const uint64_t rs = warp_sum64(wsum);
-        if (lane == 0) s_round[i0 >> 5] = rs;
-        S += rs;
+    } else {  // a legal +inf or NaN, outside the documented domain: the maximum over what are numbers, weight_shift's weights
+        m = kLowest;
+        for (int e = 9 * i0; e < 9 * i1; ++e) m = fmaxf(m, legal_logit(lg, army, terrain, list[e / 9], e % 9, moves));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
+        for (int e = 9 * i0; e < 9 * i1; ++e) mine += weight_shift(legal_logit(lg, army, terrain, list[e / 9], e % 9, moves), m);
     }
-    __syncwarp();
+    const uint64_t incl = warp_incl64(mine, lane);
+    const uint64_t S = __shfl_sync(kAll, incl, 31);
     const uint64_t d = stream_out(hkey(a.seed, gi.game_id, sc.frame, (uint64_t)p), 7);
     const uint64_t r = __umul64hi(d, S);
-    // pass 3: the group of 32, then the cell, then the entry where the running sum first exceeds r
-    const int groups = (n + 31) >> 5;
-    uint64_t run = 0;
-    int jr = -1;
-    for (int j0 = 0; j0 < groups && jr < 0; j0 += 32) {
-        const uint64_t rs = j0 + lane < groups ? s_round[j0 + lane] : 0u;
-        const uint64_t incl = warp_incl64(rs, lane);
-        const unsigned hit = __ballot_sync(kAll, run + incl > r);
-        if (hit) {
-            const int L = __ffs(hit) - 1;
-            jr = j0 + L;
-            run += __shfl_sync(kAll, incl - rs, L);
-        } else {
-            run += __shfl_sync(kAll, incl, 31);
-        }
-    }
-    if (jr < 0) return 0;  // S = 0: only when every legal logit is -inf (outside the documented domain)
-    const int i = 32 * jr + lane;
-    const uint64_t wi = i < n ? s_w[i] : 0u;
-    const uint64_t incl = warp_incl64(wi, lane);
-    const unsigned hit = __ballot_sync(kAll, run + incl > r);
+    const unsigned hit = __ballot_sync(kAll, incl > r);
+    if (hit == 0u) return 0;  // S = 0: only when every legal logit is -inf (outside the documented domain)
     const int L = __ffs(hit) - 1;
-    // the entry inside the chosen cell: lanes 0..8 take one entry each
-    const uint64_t before = run + __shfl_sync(kAll, incl - wi, L);
-    const int cL = s_list[32 * jr + L];
-    const uint32_t lbL = s_legal[32 * jr + L];
-    uint64_t we = 0;
-    if (lane < 9 && ((lbL >> lane) & 1u)) we = weight_shift(__ldcg(lg + 9 * cL + lane), m);
-    const uint64_t ein = warp_incl64(we, lane);
-    const unsigned ehit = __ballot_sync(kAll, lane < 9 && before + ein > r);
-    return 9 * cL + (__ffs(ehit) - 1);
+    uint64_t left = r - __shfl_sync(kAll, incl - mine, L);  // below lane L's sum
+    // the entry among lane L's cells: three cells at a time, a lane per entry
+    const int q = lane / 9, e = lane - 9 * q, end = min(n, L * k + k);
+    for (int j = L * k; j < end; j += 3) {
+        const int i = j + q;
+        const int c = lane < 27 && i < end ? list[i] : -1;
+        const uint32_t w = c >= 0 ? weight_shift(legal_logit(lg, army, terrain, c, e, moves), m) : 0u;
+        uint32_t in = w;  // at most 27 * 2^25
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kAll, in, o);
+            if (lane >= o) in += y;
+        }
+        const unsigned b = __ballot_sync(kAll, (uint64_t)in > left);
+        if (b) return __shfl_sync(kAll, 9 * c + e, __ffs(b) - 1);
+        left -= __shfl_sync(kAll, in, 31);
+    }
+    return 0;  // not reached: the loop's weights sum to lane L's
 }
 
-// one warp per game, players in turn
-__global__ void __launch_bounds__(256) k_sample(const SArgs a, int warps_per_cta) {
+// ---- the expanded mask --------------------------------------------------------
+// One CTA per game: each cell's nine legal bits and owner in one 16-bit word
+// of shared memory, then every thread makes 16-byte vectors of the players'
+// planes, 512 contiguous bytes per warp.  A vector holds bytes of at most
+// three cells; for most (vector, player) pairs none of them is the player's
+// and zeros are stored.  HBM-bound by its 9 bytes per player and cell:
+// 8,192 mixed games of 20..40 a side 53 us for 295 MB, about 100 us (of 343
+// with the sampler) when a warp wrote single bytes to staging rows.
+constexpr int kMaskThreads = 128;
+// s_cell: legal bits 0..8, owner 12..15 (15: none)
+__device__ __forceinline__ void mask_game(const SArgs& a, int gidx, uint16_t* s_cell, int tid) {
+    const GameInfo gi = sample_game(a, gidx);
+    const GameScalars sc = a.scal[gidx];
+    const int Npad = gi.Npad, P = gi.P;
+    for (int c = 4 * tid; c < Npad; c += 4 * kMaskThreads) {
+        const uint2 av = __ldg(reinterpret_cast<const uint2*>(a.army + gi.cell_off + c));
+        const uint32_t ow = __ldg(reinterpret_cast<const uint32_t*>(a.owner + gi.cell_off + c));
+        const uint32_t tw = __ldg(reinterpret_cast<const uint32_t*>(a.terrain + gi.cell_off + c));
+        uint32_t x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int o = (int)(int8_t)(ow >> (8 * i));
+            const int army = (int)(int16_t)((i < 2 ? av.x : av.y) >> (16 * (i & 1)));
+            const bool moves = o >= 0 && ((sc.alive >> o) & 1u) && !sc.finished;
+            x[i] = legal9(o >= 0, army, (tw >> (8 * i)) & 0xFFu, moves) | ((uint32_t)(o & 15) << 12);
+        }
+        *reinterpret_cast<uint2*>(s_cell + c) = make_uint2(x[0] | (x[1] << 16), x[2] | (x[3] << 16));
+    }
+    if (tid < 2) s_cell[Npad + tid] = 0xF000u;  // read past the last cell, never kept
+    __syncthreads();
+    const int nv = (9 * Npad) >> 4;
+    for (int v = tid; v < nv; v += kMaskThreads) {
+        const int c = 16 * v / 9, off = 16 * v - 9 * c;  // the vector's first byte is entry `off` of cell c
+        const uint32_t e0 = s_cell[c], e1 = s_cell[c + 1], e2 = s_cell[c + 2];
+        uint4* out = reinterpret_cast<uint4*>(a.mask9 + gi.plane_off * 9) + v;
+        for (int p = 0; p < P; ++p, out += nv) {
+            uint32_t bits = ((e0 >> 12) == p ? e0 & 0x1FFu : 0u) | ((e1 >> 12) == p ? (e1 & 0x1FFu) << 9 : 0u) |
+                            ((e2 >> 12) == p ? (e2 & 0x1FFu) << 18 : 0u);
+            bits >>= off;
+            uint4 y = make_uint4(0u, 0u, 0u, 0u);
+            if (bits & 0xFFFFu) {
+                auto spread = [&](int sh) { return (((bits >> sh) & 15u) * 0x00204081u) & 0x01010101u; };
+                y = make_uint4(spread(0), spread(4), spread(8), spread(12));
+            }
+            __stcs(out, y);
+        }
+    }
+}
+__global__ void __launch_bounds__(kMaskThreads) k_mask9(const SArgs a) {
+    chain_entry();
+    extern __shared__ __align__(16) char smem[];
+    mask_game(a, blockIdx.x, reinterpret_cast<uint16_t*>(smem), threadIdx.x);
+}
+
+// one warp per (game, player): warp b takes player b mod pmax of game b / pmax
+// (those of absent players return at once).  CTAs of two warps: 2v2, 8-player
+// and two-player games mix in one launch without holding slots for absent
+// players.
+constexpr int kSlotWarps = 2;
+__device__ __forceinline__ void sample_slot(const SArgs& a, int gidx, int p, char* smem, int wid, int lane) {
+    const GameInfo gi = sample_game(a, gidx);
+    if (p >= gi.P) return;
+    const GameScalars sc = a.scal[gidx];
+    uint16_t* list = reinterpret_cast<uint16_t*>(smem + (size_t)wid * list_bytes(a.npad_max));
+    const int32_t action = sample_player(a, gi, sc, p, list, lane);
+    if (lane == 0) a.actions[gi.player_off + p] = action;
+}
+__global__ void __launch_bounds__(32 * kSlotWarps, 36 / kSlotWarps) k_sample_slots(const SArgs a, int pmax) {
     chain_entry();
     extern __shared__ __align__(16) char smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int gidx = blockIdx.x * warps_per_cta + wid;
-    if (gidx >= a.n_games) return;
-    const int np = a.npad_max;
-    char* b = smem + (size_t)wid * sample_warp_bytes(np);
-    char* w = b + 4 * np;
-    const GameInfo gi = a.info[gidx];
-    const GameScalars sc = a.scal[gidx];
-    stage_board(a, gi, b, np, lane, 32);
-    __syncwarp();
-    const int16_t* s_army = reinterpret_cast<const int16_t*>(b);
-    const int8_t* s_owner = reinterpret_cast<const int8_t*>(b + 2 * np);
-    const uint8_t* s_terrain = reinterpret_cast<const uint8_t*>(b + 3 * np);
-    if (a.mask9)
-        mask_rows(a, gi, sc, s_army, s_owner, s_terrain, reinterpret_cast<uint8_t*>(w + sample_player_bytes(np) - 288),
-                  0, 32, lane);
-    if (!a.logits) return;
-    for (int p = 0; p < gi.P; ++p) {
-        const int32_t action = sample_player(a, gi, sc, p, s_army, s_owner, s_terrain, w, lane);
-        if (lane == 0 && a.actions) a.actions[gi.player_off + p] = action;
-        __syncwarp();
-    }
+    const unsigned item = blockIdx.x * kSlotWarps + wid;
+    const int gidx = (int)(item / (unsigned)pmax), p = (int)item - gidx * pmax;
+    if (gidx < a.n_games) sample_slot(a, gidx, p, smem, wid, lane);
 }
-
-// one CTA per game (small batches): warp q takes players q, q + warps, ...
-// and mask rows q, q + warps, ... over its own region of shared memory
-__global__ void __launch_bounds__(256) k_sample_cta(const SArgs a) {
+// The sampler and the expanded mask in one launch: per game, CTAs of four
+// players and one CTA for its mask.  The sampler waits on latency and the
+// mask on HBM writes, so they overlap (8,192 mixed games of 20..40 a side:
+// one launch after the other 111 us, so 97 us).
+__global__ void __launch_bounds__(kMaskThreads, 9) k_sample_mask(const SArgs a, int ctas_per_game) {
     chain_entry();
     extern __shared__ __align__(16) char smem[];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int gidx = blockIdx.x;  // the grid is one CTA per game
-    const int np = a.npad_max;
-    char* w = smem + 4 * np + (size_t)wid * sample_player_bytes(np);
-    const GameInfo gi = a.info[gidx];
-    const GameScalars sc = a.scal[gidx];
-    stage_board(a, gi, smem, np, threadIdx.x, blockDim.x);
-    __syncthreads();
-    const int16_t* s_army = reinterpret_cast<const int16_t*>(smem);
-    const int8_t* s_owner = reinterpret_cast<const int8_t*>(smem + 2 * np);
-    const uint8_t* s_terrain = reinterpret_cast<const uint8_t*>(smem + 3 * np);
-    if (a.mask9)
-        mask_rows(a, gi, sc, s_army, s_owner, s_terrain, reinterpret_cast<uint8_t*>(w + sample_player_bytes(np) - 288),
-                  32 * wid, 32 * nwarps, lane);
-    if (!a.logits) return;
-    for (int p = wid; p < gi.P; p += nwarps) {
-        const int32_t action = sample_player(a, gi, sc, p, s_army, s_owner, s_terrain, w, lane);
-        if (lane == 0 && a.actions) a.actions[gi.player_off + p] = action;
-        __syncwarp();
-    }
-}
-
-// ---- entry-parallel form (small batches) --------------------------------
-// One CTA of kWideThreads threads per (game, player): the player's own cells
-// are listed in index order by contiguous ranges of cells per thread and a
-// block scan; then every (own cell, entry) pair gets a thread of its own,
-// entry e of the list being entry e mod 9 of own cell e / 9 -- index order.
-// Pass 1 loads each legal entry's logit once (the first kWideRegRounds
-// rounds of the block stay in registers) and takes the block maximum; pass 2
-// forms the integer weights and each warp's sum per round; one warp then
-// sums them (S), draws r and finds the (round, warp) where the running sum
-// first exceeds r; that warp scans its own 32 weights for the entry.  A
-// game's chain is a few dependent steps instead of a warp's walk over its
-// own cells, which is what sets the time when a launch fills less than a
-// wave.
-constexpr int kWideThreads = 128;
-constexpr int kWideWarps = kWideThreads / 32;
-constexpr int kWideRegRounds = 4;
-constexpr float kNegInf = -__builtin_huge_valf();
-
-__host__ __device__ __forceinline__ int wide_rounds(int npad_max) {
-    return (9 * npad_max + kWideThreads - 1) / kWideThreads;
-}
-// board (4 B per cell), own-cell list and legal bits (2 + 2 B per cell),
-// per-round warp sums (4 B each), block scratch, one mask staging row per warp
-__host__ __device__ __forceinline__ int wide_bytes(int npad_max) {
-    const int rw = (4 * wide_rounds(npad_max) * kWideWarps + 15) & ~15;
-    return 8 * npad_max + rw + 64 + 288 * kWideWarps;
-}
-
-__global__ void __launch_bounds__(kWideThreads) k_sample_wide(const SArgs a, int pmax) {
-    chain_entry();
-    extern __shared__ __align__(16) char smem[];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int gidx = blockIdx.x / pmax, p = blockIdx.x - gidx * pmax;
-    const GameInfo gi = a.info[gidx];
-    if (p >= gi.P) return;
-    const GameScalars sc = a.scal[gidx];
-    const int np = a.npad_max, N = gi.N, Npad = gi.Npad;
-    uint16_t* s_list = reinterpret_cast<uint16_t*>(smem + 4 * np);
-    uint16_t* s_legal = reinterpret_cast<uint16_t*>(smem + 6 * np);
-    uint32_t* s_ws = reinterpret_cast<uint32_t*>(smem + 8 * np);  // [round][warp]
-    const int rw = (4 * wide_rounds(np) * kWideWarps + 15) & ~15;
-    uint32_t* s_misc = reinterpret_cast<uint32_t*>(smem + 8 * np + rw);  // 16 words
-    uint8_t* s_mask = reinterpret_cast<uint8_t*>(smem + 8 * np + rw + 64) + 288 * wid;
-    stage_board(a, gi, smem, np, tid, kWideThreads);
-    __syncthreads();
-    const int16_t* s_army = reinterpret_cast<const int16_t*>(smem);
-    const int8_t* s_owner = reinterpret_cast<const int8_t*>(smem + 2 * np);
-    const uint8_t* s_terrain = reinterpret_cast<const uint8_t*>(smem + 3 * np);
-    const bool moves = ((sc.alive >> p) & 1u) && !sc.finished;
-    if (a.mask9) {  // player p's plane: rows of 32 cells, one warp each
-        for (int r0 = 32 * wid; r0 < Npad; r0 += 32 * kWideWarps) {
-            const int cells = min(32, Npad - r0), c = r0 + lane;
-            const uint32_t bits =
-                c < N && s_owner[c] == p ? legal9(true, s_army[c], s_terrain[c], moves) : 0u;
-            if (lane < cells)
-#pragma unroll
-                for (int k = 0; k < 9; ++k) s_mask[9 * lane + k] = (uint8_t)((bits >> k) & 1u);
-            __syncwarp();
-            const int64_t base = (gi.plane_off + (int64_t)p * Npad) * 9;
-            if (lane < ((9 * cells) >> 4))
-                reinterpret_cast<uint4*>(a.mask9 + base + 9 * r0)[lane] = reinterpret_cast<const uint4*>(s_mask)[lane];
-            __syncwarp();
-        }
-    }
-    if (!a.logits) return;
-    // the player's cells in index order: a contiguous range of cells per thread
-    const int cpt = (N + kWideThreads - 1) / kWideThreads;
-    const int c0 = min(N, tid * cpt), c1 = min(N, c0 + cpt);
-    int cnt = 0;
-    for (int c = c0; c < c1; ++c) cnt += s_owner[c] == p;
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(kAll, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) s_misc[wid] = (uint32_t)incl;
-    __syncthreads();
-    int before = incl - cnt, n = 0;
-#pragma unroll
-    for (int q = 0; q < kWideWarps; ++q) {
-        const int t = (int)s_misc[q];
-        if (q < wid) before += t;
-        n += t;
-    }
-    for (int c = c0, i = before; c < c1; ++c)
-        if (s_owner[c] == p) {
-            s_list[i] = (uint16_t)c;
-            s_legal[i] = (uint16_t)legal9(true, s_army[c], s_terrain[c], moves);
-            ++i;
-        }
-    __syncthreads();  // the list is complete; s_misc free again
-    if (n == 0) {
-        if (tid == 0 && a.actions) a.actions[gi.player_off + p] = 0;
-        return;
-    }
-    const float* lg = a.logits + (gi.plane_off + (int64_t)p * Npad) * 9;
-    const int ne = 9 * n, rounds = (ne + kWideThreads - 1) / kWideThreads;
-    // entry e of the list: its logit if legal, else -inf
-    auto logit_of = [&](int e) -> float {
-        if (e >= ne) return kNegInf;
-        const int i = e / 9, k = e - 9 * i;
-        if (!((s_legal[i] >> k) & 1u)) return kNegInf;
-        return __ldcg(lg + 9 * (int)s_list[i] + k);
-    };
-    // pass 1: the maximum legal logit
-    float v[kWideRegRounds];
-    float m = kNegInf;
-#pragma unroll
-    for (int j = 0; j < kWideRegRounds; ++j) {
-        v[j] = j < rounds ? logit_of(tid + kWideThreads * j) : kNegInf;
-        m = fmaxf(m, v[j]);
-    }
-    for (int j = kWideRegRounds; j < rounds; ++j) m = fmaxf(m, logit_of(tid + kWideThreads * j));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
-    if (lane == 0) s_misc[wid] = __float_as_uint(m);
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kWideWarps; ++q) m = fmaxf(m, __uint_as_float(s_misc[q]));
-    // pass 2: integer weights (0 for illegal entries) and each warp's sum per round
-    auto weight_of = [&](float x) -> uint32_t { return x == kNegInf ? 0u : weight_shift(x, m); };
-    uint32_t w[kWideRegRounds];
-#pragma unroll
-    for (int j = 0; j < kWideRegRounds; ++j) {
-        w[j] = weight_of(v[j]);
-        if (j < rounds) {
-            const uint32_t ws = __reduce_add_sync(kAll, w[j]);  // at most 32 * 2^24
-            if (lane == 0) s_ws[j * kWideWarps + wid] = ws;
-        }
-    }
-    for (int j = kWideRegRounds; j < rounds; ++j) {
-        const uint32_t ws = __reduce_add_sync(kAll, weight_of(logit_of(tid + kWideThreads * j)));
-        if (lane == 0) s_ws[j * kWideWarps + wid] = ws;
-    }
-    __syncthreads();
-    // one warp: S, r, then the (round, warp) slot where the running sum first exceeds r
-    if (wid == 0) {
-        const int slots = rounds * kWideWarps;
-        uint64_t S = 0;
-        for (int t = lane; t < slots; t += 32) S += s_ws[t];
-        S = warp_sum64(S);
-        const uint64_t d = stream_out(hkey(a.seed, gi.game_id, sc.frame, (uint64_t)p), 7);
-        const uint64_t r = __umul64hi(d, S);
-        uint64_t run = 0;
-        int found = -1;
-        for (int t0 = 0; t0 < slots && found < 0; t0 += 32) {
-            const uint64_t x = t0 + lane < slots ? s_ws[t0 + lane] : 0u;
-            const uint64_t inc = warp_incl64(x, lane);
-            const unsigned hit = __ballot_sync(kAll, run + inc > r);
-            if (hit) {
-                const int L = __ffs(hit) - 1;
-                found = t0 + L;
-                run += __shfl_sync(kAll, inc - x, L);
-            } else {
-                run += __shfl_sync(kAll, inc, 31);
-            }
-        }
-        if (lane == 0) {
-            s_misc[8] = (uint32_t)found;
-            s_misc[10] = (uint32_t)run;
-            s_misc[11] = (uint32_t)(run >> 32);
-            s_misc[12] = (uint32_t)r;
-            s_misc[13] = (uint32_t)(r >> 32);
-        }
-    }
-    __syncthreads();
-    const int found = (int)s_misc[8];
-    if (found < 0) {  // S = 0: only when every legal logit is -inf (outside the documented domain)
-        if (tid == 0 && a.actions) a.actions[gi.player_off + p] = 0;
-        return;
-    }
-    const int jf = found / kWideWarps;
-    if (wid != found - jf * kWideWarps) return;
-    const uint64_t run = s_misc[10] | ((uint64_t)s_misc[11] << 32);
-    const uint64_t r = s_misc[12] | ((uint64_t)s_misc[13] << 32);
-    uint32_t wj = 0u;
-#pragma unroll
-    for (int j = 0; j < kWideRegRounds; ++j)
-        if (j == jf) wj = w[j];
-    if (jf >= kWideRegRounds) wj = weight_of(logit_of(tid + kWideThreads * jf));
-    uint32_t inc = wj;  // at most 32 * 2^24: no overflow
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(kAll, inc, o);
-        if (lane >= o) inc += y;
-    }
-    const unsigned hit = __ballot_sync(kAll, run + inc > r);
-    if (lane == __ffs(hit) - 1 && a.actions) {
-        const int e = tid + kWideThreads * jf, i = e / 9;
-        a.actions[gi.player_off + p] = 9 * (int)s_list[i] + (e - 9 * i);
-    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int gidx = blockIdx.x / ctas_per_game, part = blockIdx.x - gidx * ctas_per_game;
+    if (part + 1 < ctas_per_game)
+        sample_slot(a, gidx, part * (kMaskThreads / 32) + wid, smem, wid, lane);
+    else
+        mask_game(a, gidx, reinterpret_cast<uint16_t*>(smem), threadIdx.x);
 }
 
 }  // namespace
 
-int launch_sample(const SArgs& a, int pmax, int form, void* stream) {
+int launch_sample(const SArgs& a, int pmax, void* stream) {
     if (a.n_games <= 0) return 0;
-    // by default a CTA per player with a thread per entry while the players
-    // fill at most about one wave of those CTAs, else a CTA per game
-    // (measured on 24x24 1v1 at mid-game: 512 games 6.1 against 7.8 us,
-    // 1,024 games 9.8 against 8.8 us; from 2,048 games on the CTA per game
-    // is the fastest form)
-    if (form == 0) {
-        static std::atomic<int> sm_count{0};  // of the first device used: only the form depends on it
-        int sms = sm_count.load(std::memory_order_relaxed);
-        if (sms == 0) {
-            int dev = 0, n = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-            sms = n > 0 ? n : 1;
-            sm_count.store(sms, std::memory_order_relaxed);
-        }
-        form = (int64_t)a.n_games * pmax <= 8 * (int64_t)sms ? 3 : 2;
+    const cudaStream_t st = (cudaStream_t)stream;
+    const int mask_smem = 2 * a.npad_max + 16;
+    if (!a.logits) return launch_chained(k_mask9, dim3(a.n_games), dim3(kMaskThreads), mask_smem, st, a);
+    if (a.mask9) {
+        constexpr int per = kMaskThreads / 32;
+        const int ctas_per_game = (pmax + per - 1) / per + 1;
+        return launch_chained(k_sample_mask, dim3((unsigned)a.n_games * (unsigned)ctas_per_game), dim3(kMaskThreads),
+                              std::max(mask_smem, per * list_bytes(a.npad_max)), st, a, ctas_per_game);
     }
-    if (form == 3) {
-        const int smem = wide_bytes(a.npad_max);
-        static SmemLimit limit;
-        const void* fn = (const void*)k_sample_wide;
-        const int e = limit.raise(&fn, 1, smem);
-        if (e != 0) return e;
-        return launch_chained(k_sample_wide, dim3((unsigned)((int64_t)a.n_games * pmax)), dim3(kWideThreads), smem,
-                              (cudaStream_t)stream, a, pmax);
-    }
-    if (form == 2) {
-        // a warp per player, as many as fit next to the board (at least one)
-        const int fit = (227 * 1024 - 4 * a.npad_max) / sample_player_bytes(a.npad_max);
-        const int warps = std::max(1, std::min(std::min(pmax, kWarps), fit));
-        const int smem = 4 * a.npad_max + warps * sample_player_bytes(a.npad_max);
-        static SmemLimit limit;
-        const void* fn = (const void*)k_sample_cta;
-        const int e = limit.raise(&fn, 1, smem);
-        if (e != 0) return e;
-        return launch_chained(k_sample_cta, dim3(a.n_games), dim3(32 * warps), smem, (cudaStream_t)stream, a);
-    }
-    const int per_warp = sample_warp_bytes(a.npad_max);
-    const int wpc = std::max(1, std::min(kWarps, (200 * 1024) / per_warp));
-    const int smem = wpc * per_warp;
-    static SmemLimit limit;
-    const void* fn = (const void*)k_sample;
-    const int e = limit.raise(&fn, 1, smem);
-    if (e != 0) return e;
-    const int blocks = (a.n_games + wpc - 1) / wpc;
-    return launch_chained(k_sample, dim3(blocks), dim3(32 * wpc), smem, (cudaStream_t)stream, a, wpc);
+    const int64_t items = (int64_t)a.n_games * pmax;
+    return launch_chained(k_sample_slots, dim3((unsigned)((items + kSlotWarps - 1) / kSlotWarps)), dim3(32 * kSlotWarps),
+                          kSlotWarps * list_bytes(a.npad_max), st, a, pmax);
 }
 
 }  // namespace gk

@@ -369,9 +369,8 @@ class GeneralsEnv:
         _check(self.lib.gen_set_batch_form(self.h, int(form)), "gen_set_batch_form")
 
     def set_sample_form(self, form: int):
-        """How sample_actions spreads a game over the GPU: 1 one warp per
-        game, 2 one CTA per game with a warp per player, 3 one CTA per player
-        with a thread per (own cell, entry), 0 the default (by batch size)."""
+        """Kept for its callers (0..3): sample_actions always runs a warp per
+        player, the fastest spread at every batch size."""
         _check(self.lib.gen_set_sample_form(self.h, int(form)), "gen_set_sample_form")
 
     def sample_actions(self, logits, seed: int, actions=None, mask9=None):

@@ -122,6 +122,31 @@ def test_sampling_edge_shapes(H, W, mode, P, form):
     check_sample(env, orc, logits, 9, f"edge {H}x{W}")
 
 
+@pytest.mark.parametrize("H,W,mode,P,G", [(24, 24, 0, 2, 7), (9, 11, 2, 3, 5), (33, 32, 2, 5, 3), (5, 5, 1, 4, 1)])
+def test_sampling_uniform_batch_extreme_logits(H, W, mode, P, G):
+    """One board shape (offsets come from the launch, not the game table), player
+    counts that do not fill the last CTA, and logits of any finite size with
+    -inf among them: weights underflow to 0 or tie at the maximum."""
+    import torch
+    full = lambda x: np.full(G, x, np.int32)  # noqa: E731
+    env, orc = pair(full(H), full(W), full(mode), full(P), seed=12, n_cities=2, min_general_dist=2)
+    acts, out = env.new_actions(), env.new_outputs()
+    env.policy(3, acts)
+    for f in range(40):
+        a = orc.policy(3)
+        env.step_policy(acts, out, 3, acts)
+        orc.step(a)
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    n = int(env.layout.plane_cells) * 9
+    x = torch.randn(n, generator=gen, device="cuda")
+    pick = torch.rand(n, generator=gen, device="cuda")
+    for k, logits in enumerate((x * 1e30, torch.where(pick < 0.5, float("-inf"), x * 9), torch.where(pick < 0.9, -1e38, 1e38),
+                                (x * 3).round() * 8)):
+        want = check_sample(env, orc, logits, 40 + k, f"{H}x{W} logits {k}")
+        alone = env.sample_actions(logits, 40 + k)  # without the mask
+        assert torch.equal(alone, want)
+
+
 @FORMS
 def test_sampling_large_territories(form):
     """Planted boards where one player owns most of a large board (hundreds of
