@@ -1,7 +1,7 @@
 """Build libgenerals.so in-tree for sm_103a with nvcc (no cmake).
 
-The translation units (step kernels, C-ABI, server, feature builder,
-sampler) compile in parallel, then link into
+The translation units (step kernels per frame, multi-frame and work-list,
+C-ABI, server, feature builder, sampler) compile in parallel, then link into
 ``paper_2606_23348_gb300/_build/libgenerals.so``.
 """
 from __future__ import annotations
@@ -15,7 +15,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "libgenerals.so")
-SOURCES = ["gk_kernels.cu", "gk_capi.cu", "gk_server.cu", "gk_features.cu", "gk_sample.cu"]
+SOURCES = ["gk_kernels.cu", "gk_rollout.cu", "gk_worklist.cu", "gk_capi.cu", "gk_server.cu", "gk_features.cu", "gk_sample.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
 
