@@ -64,9 +64,8 @@ uint32_t bucket_geom(int npad_max, int nw_stride, int pmax, bool narrow) {
 }
 
 int worklist_shape(bool multi, int* cta_smem, int* ctas) {
-    // four CTAs of 8 warps per SM per frame (the register budget's limit),
-    // three in multi-frame launches; each takes an equal share of the SM's
-    // shared memory less the per-CTA reservation
+    // three CTAs of 8 warps per SM (the register budget's limit); each takes an
+    // equal share of the SM's shared memory less the per-CTA reservation
     // (the same shape with spawn options: their kernel has the same budget)
     const void* f = (const void*)worklist_kernel(multi, false);
     int dev = 0, sms = 0, smem_sm = 0, reserved = 0;
@@ -75,7 +74,7 @@ int worklist_shape(bool multi, int* cta_smem, int* ctas) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-    const int want = multi ? 3 : 4;
+    const int want = 3;
     int bytes = ((smem_sm / want - reserved - 64) / 16) * 16;  // 64: the kernel's static item slot
     if (bytes > 227 * 1024) bytes = 227 * 1024;
     // the kernel's own static slot counts against the per-CTA limit too
