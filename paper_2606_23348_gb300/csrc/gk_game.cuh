@@ -46,6 +46,7 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr int kQuadMaxCells = 576;
 constexpr int kPairMaxCells = 1024;
 constexpr int kPairMaxPlayers = 2;
+constexpr int kVisGuard = 4;  // zero words around a player's row bits: the rows above and below lie up to 64 cells away
 constexpr int kFallbackCells = 1024;  // see place_generals_bfs
 constexpr int kPlain = 0, kMountain = 1, kCastle = 2, kGeneral = 3;
 constexpr int kArmyMax = 32767;
@@ -73,6 +74,8 @@ __device__ __forceinline__ int uniform_below(uint32_t u, uint32_t n) { return (i
 // their games independently (also through divergent branches).
 template <int W>
 struct Grp {
+    static constexpr int width = W;
+    static constexpr bool kMasks = W < 32;  // legal moves kept as chunk masks, else as counts
     int lane;       // 0 .. W-1
     int shift;      // the group's first lane in the warp
     unsigned mask;  // the group's lanes
@@ -117,8 +120,10 @@ struct Smem {
     uint32_t* big;     // army >= 2
     uint32_t* col0;    // first column
     uint32_t* colL;    // last column
-    uint32_t* vis;     // [pmax][stride]
-    uint32_t* tmp;
+    // each player's seen-from-the-row bits (see fog_pass), kVisGuard zero words
+    // before and after every player's: [pmax][vstride()] from the first word on
+    uint32_t* vis;
+    uint32_t* tmp;  // scratch bitset: the first player's of vis
     // legal moves per (player, 16-cell chunk), one region in one of two forms:
     // groups narrower than a warp (two-player games, issue-bound) keep each
     // chunk's 64-bit mask (bit 4j + d: cell j towards d); a warp per game
@@ -129,7 +134,10 @@ struct Smem {
     uint8_t* cnt;      // [pmax][chunks], a warp per game (same bytes)
     int32_t* misc;     // [0..7] general cells, [8..15] land, [16..23] army
     int stride;
+    __device__ __forceinline__ int vstride() const { return stride + kVisGuard; }
 };
+// words of the vis region of a carve
+__host__ __device__ __forceinline__ int vis_region_words(int st, int pmax) { return kVisGuard + pmax * (st + kVisGuard); }
 
 // bytes of the legal-move region of a carve: masks for narrow groups, counts for a warp per game
 __host__ __device__ __forceinline__ int legal_region_bytes(int npad_max, int pmax, bool narrow) {
@@ -162,10 +170,8 @@ __device__ __forceinline__ Smem carve_dims(char* base, const int np, const int s
     w += st;
     s.colL = w;
     w += st;
-    s.vis = w;
-    w += pm * st;
-    s.tmp = w;
-    w += st;
+    s.vis = s.tmp = w + kVisGuard;
+    w += vis_region_words(st, pm);
     s.legal = reinterpret_cast<uint64_t*>(w);  // 8-byte aligned: every region above is
     s.cnt = reinterpret_cast<uint8_t*>(w);
     w += legal_region_bytes(np, pm, narrow) >> 2;  // whole 16-byte units
@@ -264,11 +270,11 @@ __device__ __forceinline__ void derive_passable(const Game& g, const Smem& s, co
 constexpr int kColWords = (kMaxSide * kMaxSide) / 32;
 __device__ __align__(16) uint32_t g_columns[kMaxSide][2][kColWords];
 
-template <int LW>
-__device__ __forceinline__ void column_pass(const Game& g, const Smem& s, const Grp<LW>& t) {
+template <class T>
+__device__ __forceinline__ void column_pass(const Game& g, const Smem& s, const T& t) {
     const uint32_t* c0 = g_columns[g.W - 1][0];
     const uint32_t* cl = g_columns[g.W - 1][1];
-    for (int w = t.lane; w < g.nw; w += LW) {
+    for (int w = t.lane; w < g.nw; w += t.width) {
         s.col0[w] = c0[w];
         s.colL[w] = cl[w];
     }
@@ -862,14 +868,14 @@ __device__ __forceinline__ uint16_t big_bits(const uint32_t (&aw)[8]) {
         b80[k] = __byte_perm(aw[2 * k] + 0x7FFE7FFEu, aw[2 * k + 1] + 0x7FFE7FFEu, 0x7531) & 0x80808080u;
     return (uint16_t)((collect_lo(b80[0], b80[1]) >> 7) | (collect_lo(b80[2], b80[3]) << 1));
 }
-template <int LW>
-__device__ __forceinline__ uint32_t total_saturated(uint32_t sat, bool grow, const Grp<LW>& t) {
+template <class T>
+__device__ __forceinline__ uint32_t total_saturated(uint32_t sat, bool grow, const T& t) {
     return grow && t.any(sat != 0u) ? t.reduce_add(sat) : 0u;
 }
 
 // up to PT players at once
-template <int PT, int LW>
-__device__ uint32_t chunk_pass(const Game& g, const Smem& s, bool grow_s, bool grow_p, const Grp<LW>& t) {
+template <int PT, class T>
+__device__ uint32_t chunk_pass(const Game& g, const Smem& s, bool grow_s, bool grow_p, const T& t) {
     const int P = g.P, nch = g.nch, st2 = 2 * s.stride;
     uint32_t sat = 0;
     uint32_t arm[PT], land[PT / 2];  // land: two players' counts per word
@@ -879,7 +885,7 @@ __device__ uint32_t chunk_pass(const Game& g, const Smem& s, bool grow_s, bool g
     for (int p = 0; p < PT / 2; ++p) land[p] = 0;
     uint16_t* own16 = reinterpret_cast<uint16_t*>(s.own);
     uint16_t* big16 = reinterpret_cast<uint16_t*>(s.big);
-    for (int ch = t.lane; ch < nch; ch += LW) {
+    for (int ch = t.lane; ch < nch; ch += t.width) {
         const int c0 = ch << 4;
         const uint4 O = *reinterpret_cast<const uint4*>(s.owner + c0);
         const uint32_t ow[4] = {O.x, O.y, O.z, O.w};
@@ -925,13 +931,13 @@ __device__ uint32_t chunk_pass(const Game& g, const Smem& s, bool grow_s, bool g
 
 // the players one after another: more shared-memory loads, but few values
 // live at once
-template <int LW>
-__device__ uint32_t chunk_pass_in_turn(const Game& g, const Smem& s, bool grow_s, bool grow_p, const Grp<LW>& t) {
+template <class T>
+__device__ uint32_t chunk_pass_in_turn(const Game& g, const Smem& s, bool grow_s, bool grow_p, const T& t) {
     const int P = g.P, nch = g.nch, st2 = 2 * s.stride;
     uint32_t sat = 0;
     uint16_t* own16 = reinterpret_cast<uint16_t*>(s.own);
     uint16_t* big16 = reinterpret_cast<uint16_t*>(s.big);
-    for (int ch = t.lane; ch < nch; ch += LW) {
+    for (int ch = t.lane; ch < nch; ch += t.width) {
         uint32_t aw[8];
         grown_armies(s, ch << 4, grow_s, grow_p, aw, sat);
         big16[ch] = big_bits(aw);
@@ -942,7 +948,7 @@ __device__ uint32_t chunk_pass_in_turn(const Game& g, const Smem& s, bool grow_s
         const uint32_t p4 = 0x01010101u * (uint32_t)p;
         uint32_t arm = 0, land = 0;  // arm: times 128 (at most 8 chunks of 16 armies per lane)
 #pragma unroll 1
-        for (int ch = t.lane; ch < nch; ch += LW) {
+        for (int ch = t.lane; ch < nch; ch += t.width) {
             const int c0 = ch << 4;
             const uint4 O = *reinterpret_cast<const uint4*>(s.owner + c0);
             const uint4 A0 = *reinterpret_cast<const uint4*>(s.army + c0);
@@ -978,54 +984,64 @@ __device__ uint32_t chunk_pass_in_turn(const Game& g, const Smem& s, bool grow_s
 // slower (4,096 30x30 free-for-all games: 51.3 against 50.5 us), and a
 // multi-frame kernel that never runs them is faster without their code (64
 // frames of 1,024 1v1 games: 293 against 286 us).
-template <bool IN_TURN, int LW>
-__device__ __forceinline__ uint32_t cell_pass(const Game& g, const Smem& s, bool grow_s, bool grow_p, const Grp<LW>& t) {
-    if constexpr (LW < 32) {  // groups narrower than a warp only run games of at most kPairMaxPlayers
+template <bool IN_TURN, class T>
+__device__ __forceinline__ uint32_t cell_pass(const Game& g, const Smem& s, bool grow_s, bool grow_p, const T& t) {
+    if constexpr (T::kMasks) {  // groups narrower than a warp only run games of at most kPairMaxPlayers
         static_assert(kPairMaxPlayers == 2, "narrow groups compile the two-player cell pass only");
-        return chunk_pass<2, LW>(g, s, grow_s, grow_p, t);
+        return chunk_pass<2, T>(g, s, grow_s, grow_p, t);
     } else {
-        if (g.P <= 2) return chunk_pass<2, LW>(g, s, grow_s, grow_p, t);
-        if (g.P <= 4) return chunk_pass<4, LW>(g, s, grow_s, grow_p, t);
+        if (g.P <= 2) return chunk_pass<2, T>(g, s, grow_s, grow_p, t);
+        if (g.P <= 4) return chunk_pass<4, T>(g, s, grow_s, grow_p, t);
         if constexpr (IN_TURN)
-            return chunk_pass_in_turn<LW>(g, s, grow_s, grow_p, t);
+            return chunk_pass_in_turn(g, s, grow_s, grow_p, t);
         else
-            return chunk_pass<8, LW>(g, s, grow_s, grow_p, t);
+            return chunk_pass<8, T>(g, s, grow_s, grow_p, t);
     }
 }
 
 // ---- fog: 3x3 dilation of the (team) ownership bitset (Sec. IV-B) ----------
-template <int LW>
-__device__ void fog_pass(const Game& g, const Smem& s, uint32_t alive, const Grp<LW>& t) {
-    const int N = g.N, W = g.W, nw = g.nw, st = s.stride;
-    const int q = W >> 5, sh = W & 31;
-    const bool team = g.mode == 1;
-    for (int p = 0; p < g.P; ++p) {
-        const uint32_t* own = s.own + p * st;
-        const uint32_t* ally = s.own + (p ^ 1) * st;
-        for (int w = t.lane; w < nw; w += LW) {
-            const uint32_t mine = own[w];
-            const uint32_t T = mine | (team ? ally[w] : 0u);
-            const uint32_t Tm = (w > 0) ? (own[w - 1] | (team ? ally[w - 1] : 0u)) : 0u;
-            const uint32_t Tp = (w + 1 < nw) ? (own[w + 1] | (team ? ally[w + 1] : 0u)) : 0u;
-            const uint32_t L = (T << 1) | (Tm >> 31);  // bit c <- cell c-1
-            const uint32_t R = (T >> 1) | (Tp << 31);  // bit c <- cell c+1
-            s.tmp[w] = (T | (L & ~s.col0[w]) | (R & ~s.colL[w])) & valid_bits(N, w);
-        }
-        t.sync();
-        const bool seeing = (alive >> p) & 1u;
-        for (int w = t.lane; w < nw; w += LW) {
-            const uint32_t h = s.tmp[w];
-            // bit c <- cell c - W (row above) and cell c + W (row below)
-            const int wa = w - q;
-            uint32_t up = (wa >= 0 ? s.tmp[wa] << sh : 0u);
-            if (sh && wa - 1 >= 0) up |= s.tmp[wa - 1] >> (32 - sh);
-            const int wb = w + q;
-            uint32_t dn = (wb < nw ? s.tmp[wb] >> sh : 0u);
-            if (sh && wb + 1 < nw) dn |= s.tmp[wb + 1] << (32 - sh);
-            s.vis[p * st + w] = seeing ? ((h | up | dn) & valid_bits(N, w)) : 0u;
-        }
-        t.sync();
+// This pass widens each player's (team's) cells by one column to either side;
+// output_pass joins the row above and below as it reads a chunk's bits, for
+// which the words around a player's are zero (zero_guards).  Words of all
+// players share one loop, so that narrow groups fill their lanes.  Against a
+// second pass over the words for the rows and a loop per player: step of
+// 65,536 24x24 1v1 games 129.2 -> 120.9 us, of 32,768 mixed games 218.6 ->
+// 201.2 us, 16 frames of 32,768 ragged games 870 -> 828 us.
+template <class T>
+__device__ __forceinline__ void zero_guards(const Game& g, const Smem& s, const T& t) {
+    const int vs = s.vstride();
+    if (t.lane < kVisGuard) s.vis[t.lane - kVisGuard] = 0u;
+    for (int i = t.lane; i < g.P * 2 * kVisGuard; i += t.width) {
+        const int p = i / (2 * kVisGuard), k = i & (2 * kVisGuard - 1);
+        // past the game's own words, and past those of the carve's largest board (the next player's front)
+        s.vis[p * vs + (k < kVisGuard ? g.nw + k : s.stride + k - kVisGuard)] = 0u;
     }
+}
+template <class T>
+__device__ __forceinline__ void fog_pass(const Game& g, const Smem& s, uint32_t alive, const T& t) {
+    const int nw = g.nw, st = s.stride, vs = s.vstride();
+    const bool team = g.mode == 1;
+    int p = 0, w = t.lane;
+    while (p < g.P && w >= nw) {
+        w -= nw;
+        ++p;
+    }
+    while (p < g.P) {
+        const uint32_t* own = s.own + p * st + w;
+        const uint32_t* ally = s.own + (p ^ 1) * st + w;
+        const uint32_t T0 = own[0] | (team ? ally[0] : 0u);
+        const uint32_t Tm = w > 0 ? own[-1] | (team ? ally[-1] : 0u) : 0u;
+        const uint32_t Tp = w + 1 < nw ? own[1] | (team ? ally[1] : 0u) : 0u;
+        const uint32_t L = __funnelshift_l(Tm, T0, 1);  // bit c <- cell c-1
+        const uint32_t R = __funnelshift_r(T0, Tp, 1);  // bit c <- cell c+1
+        s.vis[p * vs + w] = ((alive >> p) & 1u) ? T0 | (L & ~s.col0[w]) | (R & ~s.colL[w]) : 0u;
+        w += t.width;
+        while (p < g.P && w >= nw) {
+            w -= nw;
+            ++p;
+        }
+    }
+    t.sync();
 }
 
 // 4 bits -> 4 bytes of 0x01
@@ -1057,10 +1073,13 @@ __device__ __forceinline__ uint64_t chunk_legal64(const Smem& s, int p, int ch) 
 
 // ---- observation + mask chunks of 16 cells (Sec. IV-B, App. A, Sec. IV-G) --
 // WRITE: store the planes; COUNT: legal (cell, direction) pairs per chunk.
-template <bool WRITE, bool COUNT, int LW>
-__device__ void output_pass(const KArgs& a, const Game& g, const Smem& s, uint32_t alive, bool finished, const Grp<LW>& t,
+template <bool WRITE, bool COUNT, class T>
+__device__ void output_pass(const KArgs& a, const Game& g, const Smem& s, uint32_t alive, bool finished, const T& t,
                             int64_t frame_off) {
-    const int nch = g.nch, st = s.stride, P = g.P;
+    const int nch = g.nch, st = s.stride, vs = s.vstride(), P = g.P;
+    // a row up or down in 16-cell units and a shift
+    const int ua = (g.W + 15) >> 4, us = 16 * ua - g.W, da = g.W >> 4, ds = g.W & 15;
+    const uint32_t tail = (1u << (((g.N - 1) & 15) + 1)) - 1u;  // the last chunk's cells on the board
     int p = 0, ch = t.lane;
     while (p < P && ch >= nch) {
         ch -= nch;
@@ -1080,7 +1099,7 @@ __device__ void output_pass(const KArgs& a, const Game& g, const Smem& s, uint32
             om[k] = dpb & (spread4((mv >> (4 * k)) & 15u) * 0xFFu);
         }
         if (COUNT) {
-            if (LW < 32) {
+            if (T::kMasks) {
                 // the chunk's legal moves as 64 bits: 4 per cell in (cell, direction) order
                 const uint32_t lo = nibbles16(om[0]) | (nibbles16(om[1]) << 16);
                 const uint32_t hi = nibbles16(om[2]) | (nibbles16(om[3]) << 16);
@@ -1092,7 +1111,10 @@ __device__ void output_pass(const KArgs& a, const Game& g, const Smem& s, uint32
             }
         }
         if (WRITE) {
-            const uint32_t vis16 = (s.vis[p * st + wi] >> sh) & 0xFFFFu;
+            const uint16_t* h = reinterpret_cast<const uint16_t*>(s.vis + p * vs) + ch;
+            const uint32_t up = ((uint32_t)h[-ua] | ((uint32_t)h[1 - ua] << 16)) >> us;  // cells c0 - W ..
+            const uint32_t dn = ((uint32_t)h[da] | ((uint32_t)h[da + 1] << 16)) >> ds;   // cells c0 + W ..
+            const uint32_t vis16 = (h[0] | up | dn) & (ch == nch - 1 ? tail : 0xFFFFu);
             const uint4 A0 = *reinterpret_cast<const uint4*>(s.army + c0);
             const uint4 A1 = *reinterpret_cast<const uint4*>(s.army + c0 + 8);
             const uint4 O = *reinterpret_cast<const uint4*>(s.owner + c0);
@@ -1120,7 +1142,7 @@ __device__ void output_pass(const KArgs& a, const Game& g, const Smem& s, uint32
             __stcs(reinterpret_cast<uint4*>(a.obs_vis + off), make_uint4(ov[0], ov[1], ov[2], ov[3]));
             __stcs(reinterpret_cast<uint4*>(a.mask + off), make_uint4(om[0], om[1], om[2], om[3]));
         }
-        ch += LW;
+        ch += t.width;
         while (p < P && ch >= nch) {
             ch -= nch;
             ++p;
@@ -1241,8 +1263,8 @@ __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
                  "l"(gmem)
                  : "memory");
 }
-template <int LW>
-__device__ __forceinline__ void board_issue(const KArgs& a, const Game& g, const Smem& s, const Grp<LW>& t) {
+template <class T>
+__device__ __forceinline__ void board_issue(const KArgs& a, const Game& g, const Smem& s, const T& t) {
     const int n16 = g.Npad >> 4;  // 16-byte vectors per int8 plane
     const uint4* ga = reinterpret_cast<const uint4*>(a.army + g.cell_off);
     const uint4* go = reinterpret_cast<const uint4*>(a.owner + g.cell_off);
@@ -1250,8 +1272,8 @@ __device__ __forceinline__ void board_issue(const KArgs& a, const Game& g, const
     uint4* sa = reinterpret_cast<uint4*>(s.army);
     uint4* so = reinterpret_cast<uint4*>(s.owner);
     uint4* st = reinterpret_cast<uint4*>(s.terrain);
-    for (int v = t.lane; v < 2 * n16; v += LW) cp_async16(sa + v, ga + v);
-    for (int v = t.lane; v < n16; v += LW) {
+    for (int v = t.lane; v < 2 * n16; v += t.width) cp_async16(sa + v, ga + v);
+    for (int v = t.lane; v < n16; v += t.width) {
         cp_async16(so + v, go + v);
         cp_async16(st + v, gt + v);
     }
@@ -1261,20 +1283,20 @@ __device__ __forceinline__ void board_issue(const KArgs& a, const Game& g, const
         // both table rows are 8-byte aligned, the region holds an even count)
         const uint32_t* c0 = g_columns[g.W - 1][0];
         const uint32_t* cl = g_columns[g.W - 1][1];
-        for (int v = t.lane; 2 * v < g.nw; v += LW) {
+        for (int v = t.lane; 2 * v < g.nw; v += t.width) {
             cp_async8(s.col0 + 2 * v, c0 + 2 * v);
             cp_async8(s.colL + 2 * v, cl + 2 * v);
         }
     }
 }
-template <int LW>
-__device__ __forceinline__ void board_wait(const Grp<LW>& t) {
+template <class T>
+__device__ __forceinline__ void board_wait(const T& t) {
     asm volatile("cp.async.wait_all;" ::: "memory");
     t.sync();
 }
 
-template <int LW>
-__device__ __forceinline__ void store_board(const KArgs& a, const Game& g, const Smem& s, const Grp<LW>& t) {
+template <class T>
+__device__ __forceinline__ void store_board(const KArgs& a, const Game& g, const Smem& s, const T& t) {
     const int n16 = g.Npad >> 4;
     uint4* ga = reinterpret_cast<uint4*>(a.army + g.cell_off);
     uint4* go = reinterpret_cast<uint4*>(a.owner + g.cell_off);
@@ -1282,8 +1304,8 @@ __device__ __forceinline__ void store_board(const KArgs& a, const Game& g, const
     const uint4* sa = reinterpret_cast<const uint4*>(s.army);
     const uint4* so = reinterpret_cast<const uint4*>(s.owner);
     const uint4* st = reinterpret_cast<const uint4*>(s.terrain);
-    for (int v = t.lane; v < 2 * n16; v += LW) ga[v] = sa[v];
-    for (int v = t.lane; v < n16; v += LW) {
+    for (int v = t.lane; v < 2 * n16; v += t.width) ga[v] = sa[v];
+    for (int v = t.lane; v < n16; v += t.width) {
         go[v] = so[v];
         gt[v] = st[v];
     }
@@ -1324,9 +1346,9 @@ __device__ __forceinline__ void finish_frame(const KArgs& a, const Game& g, cons
             }
         }
         if (a.next_actions)
-            output_pass<true, true, LW>(a, g, s, alive, fin, t, poff);
+            output_pass<true, true>(a, g, s, alive, fin, t, poff);
         else
-            output_pass<true, false, LW>(a, g, s, alive, fin, t, poff);
+            output_pass<true, false>(a, g, s, alive, fin, t, poff);
         if constexpr (!MULTI) {
             if (t.lane < g.P) {
                 a.reward[soff + g.player_off + t.lane] = my_reward;
@@ -1336,7 +1358,7 @@ __device__ __forceinline__ void finish_frame(const KArgs& a, const Game& g, cons
             if (t.lane == 0) a.done[(int64_t)f * a.game_stride + gidx] = (uint8_t)done;
         }
     } else if (a.next_actions) {
-        output_pass<false, true, LW>(a, g, s, alive, fin, t, 0);
+        output_pass<false, true>(a, g, s, alive, fin, t, 0);
     }
     if (a.next_actions) my_act = policy_pass<!MULTI, LW>(a, g, s, alive, fin, frame, game_id_of<UNI>(a, gidx), t);
 }
@@ -1376,6 +1398,7 @@ __device__ __noinline__ void new_map(const KArgs& a, int gidx, char* warp_base, 
     const Grp<LW> t(warp_lane);
     const Game g = group_game<LW>(game_of<UNI>(a, gidx));
     const Smem s = carve_geom(warp_base, geom);
+    if (a.op != OP_STEP && a.do_outputs) zero_guards(g, s, t);  // the step has set them
     generate_body<LW, SPAWN>(a, g, s, game_id_of<UNI>(a, gidx), epoch, t);
     const uint32_t alive = (1u << g.P) - 1u;
     cell_pass<true>(g, s, false, false, t);
@@ -1410,6 +1433,7 @@ __device__ __forceinline__ void run_game(const KArgs& a, const Smem& s, char* wa
     }
     // every global load of the step is issued here, before any is used
     board_issue(a, g, s, t);
+    if (a.do_outputs) zero_guards(g, s, t);
     s0 = *reinterpret_cast<const uint4*>(sc);
     s1 = *(reinterpret_cast<const uint4*>(sc) + 1);
     // player `lane`'s action for the next step (frame 0: from the caller)

@@ -102,9 +102,11 @@ int launch_worklist(const KArgs& a, const WArgs& w, int cta_smem, int ctas, void
 
 int warp_smem_bytes(int npad_max, int pmax, int* nw_stride, bool narrow) {
     int nw = (npad_max + 31) / 32;
-    nw = (nw + 1) & ~1;  // even: the carve stays a multiple of 16 bytes
+    nw = (nw + 1) & ~1;  // even: the regions stay 8-byte aligned
     if (nw_stride) *nw_stride = nw;
-    return 4 * npad_max + 4 * nw * (2 * pmax + 4) + legal_region_bytes(npad_max, pmax, narrow) + 4 * 24;
+    const int bytes = 4 * npad_max + 4 * (nw * (pmax + 3) + vis_region_words(nw, pmax)) +
+                      legal_region_bytes(npad_max, pmax, narrow) + 4 * 24;
+    return (bytes + 15) & ~15;  // the next group's board is copied 16 bytes at a time
 }
 
 int max_resident_ctas(int warps_per_cta, int smem_bytes, int* out) {
