@@ -460,8 +460,8 @@ int build_worklist(gen_env* e) {
     for (size_t i = 0; i < nb; ++i) {
         const Bucket& b = e->buckets[i];
         geoms[i].lw = (b.pmax <= 2 && b.npad_max <= 1024 && e->lane_groups != 1) ? 16 : 32;
-        geoms[i].group_smem = gk::warp_smem_bytes(b.npad_max, b.pmax, nullptr, geoms[i].lw < 32);
-        geoms[i].geom = gk::bucket_geom(b.npad_max, b.nw_stride, b.pmax, geoms[i].lw < 32);
+        geoms[i].group_smem = gk::warp_smem_bytes(b.npad_max, b.pmax, nullptr);
+        geoms[i].geom = gk::bucket_geom(b.npad_max, b.nw_stride, b.pmax);
         geoms[i].pad = 0;
     }
     if (!e->d_geoms) {

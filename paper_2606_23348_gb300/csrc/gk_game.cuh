@@ -75,7 +75,6 @@ __device__ __forceinline__ int uniform_below(uint32_t u, uint32_t n) { return (i
 template <int W>
 struct Grp {
     static constexpr int width = W;
-    static constexpr bool kMasks = W < 32;  // legal moves kept as chunk masks, else as counts
     int lane;       // 0 .. W-1
     int shift;      // the group's first lane in the warp
     unsigned mask;  // the group's lanes
@@ -124,14 +123,7 @@ struct Smem {
     // before and after every player's: [pmax][vstride()] from the first word on
     uint32_t* vis;
     uint32_t* tmp;  // scratch bitset: the first player's of vis
-    // legal moves per (player, 16-cell chunk), one region in one of two forms:
-    // groups narrower than a warp (two-player games, issue-bound) keep each
-    // chunk's 64-bit mask (bit 4j + d: cell j towards d); a warp per game
-    // keeps only its count of legal pairs (a byte), which keeps 8-player
-    // carves small, and the policy rebuilds the selected chunk's mask from
-    // the board
-    uint64_t* legal;   // [pmax][chunks], narrow groups
-    uint8_t* cnt;      // [pmax][chunks], a warp per game (same bytes)
+    uint8_t* cnt;      // [pmax][chunks]: legal (cell, direction) pairs of a player's 16-cell chunk
     int32_t* misc;     // [0..7] general cells, [8..15] land, [16..23] army
     int stride;
     __device__ __forceinline__ int vstride() const { return stride + kVisGuard; }
@@ -139,24 +131,18 @@ struct Smem {
 // words of the vis region of a carve
 __host__ __device__ __forceinline__ int vis_region_words(int st, int pmax) { return kVisGuard + pmax * (st + kVisGuard); }
 
-// bytes of the legal-move region of a carve: masks for narrow groups, counts for a warp per game
-__host__ __device__ __forceinline__ int legal_region_bytes(int npad_max, int pmax, bool narrow) {
-    return narrow ? 8 * pmax * (npad_max >> 4) : ((pmax * (npad_max >> 4) + 15) & ~15);
+__host__ __device__ __forceinline__ int count_region_bytes(int npad_max, int pmax) {
+    return (pmax * (npad_max >> 4) + 15) & ~15;
 }
 
 // A group's shared-memory geometry packed in one word: padded cells of the
-// largest board (13 bits), bitset stride in words (8 bits), players (4 bits),
-// and whether the group is narrower than a warp (bit 25: the mask form of
-// the legal-move region).
-__host__ __device__ __forceinline__ uint32_t pack_geom(int npad_max, int nw_stride, int pmax, bool narrow) {
-    return (uint32_t)npad_max | ((uint32_t)nw_stride << 13) | ((uint32_t)pmax << 21) | (narrow ? 1u << 25 : 0u);
+// largest board (13 bits), bitset stride in words (8 bits), players (4 bits).
+__host__ __device__ __forceinline__ uint32_t pack_geom(int npad_max, int nw_stride, int pmax) {
+    return (uint32_t)npad_max | ((uint32_t)nw_stride << 13) | ((uint32_t)pmax << 21);
 }
-template <int LW>
-__device__ __forceinline__ uint32_t geom_of(const KArgs& a) {
-    return pack_geom(a.npad_max, a.nw_stride, a.pmax, LW < 32);
-}
+__device__ __forceinline__ uint32_t geom_of(const KArgs& a) { return pack_geom(a.npad_max, a.nw_stride, a.pmax); }
 
-__device__ __forceinline__ Smem carve_dims(char* base, const int np, const int st, const int pm, const bool narrow) {
+__device__ __forceinline__ Smem carve_dims(char* base, const int np, const int st, const int pm) {
     Smem s;
     s.army = reinterpret_cast<int16_t*>(base);
     s.owner = reinterpret_cast<int8_t*>(base + 2 * np);
@@ -172,21 +158,18 @@ __device__ __forceinline__ Smem carve_dims(char* base, const int np, const int s
     w += st;
     s.vis = s.tmp = w + kVisGuard;
     w += vis_region_words(st, pm);
-    s.legal = reinterpret_cast<uint64_t*>(w);  // 8-byte aligned: every region above is
     s.cnt = reinterpret_cast<uint8_t*>(w);
-    w += legal_region_bytes(np, pm, narrow) >> 2;  // whole 16-byte units
+    w += count_region_bytes(np, pm) >> 2;
     s.misc = reinterpret_cast<int32_t*>(w);
     s.stride = st;
     return s;
 }
 __device__ __forceinline__ Smem carve_geom(char* base, uint32_t geom) {
-    return carve_dims(base, (int)(geom & 0x1FFFu), (int)((geom >> 13) & 0xFFu), (int)((geom >> 21) & 0xFu),
-                      ((geom >> 25) & 1u) != 0u);
+    return carve_dims(base, (int)(geom & 0x1FFFu), (int)((geom >> 13) & 0xFFu), (int)((geom >> 21) & 0xFu));
 }
 // the launch's own geometry, straight from the kernel parameters
-template <int LW>
 __device__ __forceinline__ Smem carve(char* base, const KArgs& a) {
-    return carve_dims(base, a.npad_max, a.nw_stride, a.pmax, LW < 32);
+    return carve_dims(base, a.npad_max, a.nw_stride, a.pmax);
 }
 
 struct Game {
@@ -986,7 +969,7 @@ __device__ uint32_t chunk_pass_in_turn(const Game& g, const Smem& s, bool grow_s
 // frames of 1,024 1v1 games: 293 against 286 us).
 template <bool IN_TURN, class T>
 __device__ __forceinline__ uint32_t cell_pass(const Game& g, const Smem& s, bool grow_s, bool grow_p, const T& t) {
-    if constexpr (T::kMasks) {  // groups narrower than a warp only run games of at most kPairMaxPlayers
+    if constexpr (T::width < 32) {  // groups narrower than a warp only run games of at most kPairMaxPlayers
         static_assert(kPairMaxPlayers == 2, "narrow groups compile the two-player cell pass only");
         return chunk_pass<2, T>(g, s, grow_s, grow_p, t);
     } else {
@@ -1099,16 +1082,9 @@ __device__ void output_pass(const KArgs& a, const Game& g, const Smem& s, uint32
             om[k] = dpb & (spread4((mv >> (4 * k)) & 15u) * 0xFFu);
         }
         if (COUNT) {
-            if (T::kMasks) {
-                // the chunk's legal moves as 64 bits: 4 per cell in (cell, direction) order
-                const uint32_t lo = nibbles16(om[0]) | (nibbles16(om[1]) << 16);
-                const uint32_t hi = nibbles16(om[2]) | (nibbles16(om[3]) << 16);
-                s.legal[p * nch + ch] = ((uint64_t)hi << 32) | lo;
-            } else {
-                // legal (cell, direction) pairs of the chunk: the low nibble of each mask byte
-                s.cnt[p * nch + ch] = (uint8_t)(__popc(om[0] & 0x0F0F0F0Fu) + __popc(om[1] & 0x0F0F0F0Fu) +
-                                                __popc(om[2] & 0x0F0F0F0Fu) + __popc(om[3] & 0x0F0F0F0Fu));
-            }
+            // legal pairs: either nibble of each mask byte, two words' side by side
+            s.cnt[p * nch + ch] = (uint8_t)(__popc((om[0] & 0x0F0F0F0Fu) | (om[1] & 0xF0F0F0F0u)) +
+                                            __popc((om[2] & 0x0F0F0F0Fu) | (om[3] & 0xF0F0F0F0u)));
         }
         if (WRITE) {
             const uint16_t* h = reinterpret_cast<const uint16_t*>(s.vis + p * vs) + ch;
@@ -1172,7 +1148,6 @@ template <bool DIRECT, int LW>
 __device__ int32_t policy_pass(const KArgs& a, const Game& g, const Smem& s, uint32_t alive, bool finished,
                                uint32_t frame, uint64_t gid, const Grp<LW>& t) {
     const int nch = g.nch;
-    constexpr bool masks = LW < 32;
     const int cpl = (nch + LW - 1) / LW;  // consecutive chunks per lane
     const int c_lo = t.lane * cpl;
     const int c_hi = min(c_lo + cpl, nch);
@@ -1185,13 +1160,8 @@ __device__ int32_t policy_pass(const KArgs& a, const Game& g, const Smem& s, uin
     for (int p0 = 0; p0 < g.P; p0 += 2) {
         uint32_t mine = 0;
         for (int c = c_lo; c < c_hi; ++c) {
-            if (masks) {
-                mine += __popcll(s.legal[p0 * nch + c]);
-                if (p0 + 1 < g.P) mine += (uint32_t)__popcll(s.legal[(p0 + 1) * nch + c]) << 16;
-            } else {
-                mine += s.cnt[p0 * nch + c];
-                if (p0 + 1 < g.P) mine += (uint32_t)s.cnt[(p0 + 1) * nch + c] << 16;
-            }
+            mine += s.cnt[p0 * nch + c];
+            if (p0 + 1 < g.P) mine += (uint32_t)s.cnt[(p0 + 1) * nch + c] << 16;
         }
         const uint32_t incl2 = warp_incl_scan(mine, t);
         const uint32_t total2 = t.shfl(incl2, LW - 1);
@@ -1217,13 +1187,12 @@ __device__ int32_t policy_pass(const KArgs& a, const Game& g, const Smem& s, uin
     int32_t action = 0;
     if (my_lane >= 0 && !finished && ((alive >> t.lane) & 1u)) {
         for (int c = my_lane * cpl; c < nch; ++c) {
-            const uint64_t mk = masks ? s.legal[t.lane * nch + c] : 0ull;
-            const uint32_t n = masks ? (uint32_t)__popcll(mk) : (uint32_t)s.cnt[t.lane * nch + c];
+            const uint32_t n = s.cnt[t.lane * nch + c];
             if (my_rank >= n) {
                 my_rank -= n;
                 continue;
             }
-            const uint64_t m = masks ? mk : chunk_legal64(s, t.lane, c);
+            const uint64_t m = chunk_legal64(s, t.lane, c);
             uint32_t x = (uint32_t)m;
             int bit = 0;
             const uint32_t nlo = __popc(x);
@@ -1426,7 +1395,7 @@ __device__ __forceinline__ void run_game(const KArgs& a, const Smem& s, char* wa
                 s1 = *(reinterpret_cast<const uint4*>(sc) + 1);
                 s0.z += 1;
             }
-            new_map<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of<LW>(a), t.lane + t.shift, s0.y, s0.z, s1.y, s1.z,
+            new_map<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of(a), t.lane + t.shift, s0.y, s0.z, s1.y, s1.z,
                              s1.w, 0.0f, 0u);
             return;
         }
@@ -1507,11 +1476,11 @@ __device__ __forceinline__ void run_game(const KArgs& a, const Smem& s, char* wa
                 if (a.auto_reset) {
                     epoch += 1;
                     if constexpr (!MULTI) {
-                        new_map<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of<LW>(a), t.lane + t.shift, frame + 1,
+                        new_map<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of(a), t.lane + t.shift, frame + 1,
                                          epoch, invalid, saturated, err, my_reward, done);
                         return;
                     } else {
-                        generate<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of<LW>(a),
+                        generate<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of(a),
                                                  game_id_of<UNI>(a, gidx), epoch, t.lane + t.shift);
                         turn = 0;
                         alive = (1u << g.P) - 1u;
@@ -1558,7 +1527,7 @@ __global__ void __launch_bounds__(256, MULTI ? 3 : 4) k_generals(const KArgs a) 
     const int grp = (threadIdx.x >> 5) * kGroups + wl / LW;  // group in the CTA
     const int gpc = (blockDim.x >> 5) * kGroups;                                // groups per CTA
     char* warp_base = smem_raw + grp * a.warp_smem;
-    const Smem s = carve<LW>(warp_base, a);
+    const Smem s = carve(warp_base, a);
     if constexpr (!MULTI) {  // the grid covers every item
         const int item = blockIdx.x * gpc + grp;
         if (item >= a.n_items) return;

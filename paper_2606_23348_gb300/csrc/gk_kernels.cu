@@ -59,8 +59,8 @@ int allow_max_smem() {
     return limit.raise(fns, 15, 227 * 1024);
 }
 
-uint32_t bucket_geom(int npad_max, int nw_stride, int pmax, bool narrow) {
-    return pack_geom(npad_max, nw_stride, pmax, narrow);
+uint32_t bucket_geom(int npad_max, int nw_stride, int pmax) {
+    return pack_geom(npad_max, nw_stride, pmax);
 }
 
 int worklist_shape(bool multi, int* cta_smem, int* ctas) {
@@ -100,12 +100,12 @@ int launch_worklist(const KArgs& a, const WArgs& w, int cta_smem, int ctas, void
     return launch_chained(worklist_kernel(multi, has_spawn_options(a)), dim3(grid), dim3(256), cta_smem, st, a, w);
 }
 
-int warp_smem_bytes(int npad_max, int pmax, int* nw_stride, bool narrow) {
+int warp_smem_bytes(int npad_max, int pmax, int* nw_stride) {
     int nw = (npad_max + 31) / 32;
     nw = (nw + 1) & ~1;  // even: the regions stay 8-byte aligned
     if (nw_stride) *nw_stride = nw;
     const int bytes = 4 * npad_max + 4 * (nw * (pmax + 3) + vis_region_words(nw, pmax)) +
-                      legal_region_bytes(npad_max, pmax, narrow) + 4 * 24;
+                      count_region_bytes(npad_max, pmax) + 4 * 24;
     return (bytes + 15) & ~15;  // the next group's board is copied 16 bytes at a time
 }
 
@@ -223,18 +223,13 @@ int launch_step(const KArgs& a, int warps_per_cta, int max_ctas, void* stream) {
     const bool large = a.n_items >= (multi ? 24 : 12) * sms;
     const bool small = a.pmax <= kPairMaxPlayers && (a.lane_groups == 2 || (a.lane_groups == 0 && large));
     const int wcap = warps_per_cta > 0 ? warps_per_cta : 1;  // the fixed shape must fit too
-    // narrow groups keep their legal moves as chunk masks: a larger carve
-    const int ws_narrow = small ? warp_smem_bytes(a.npad_max, a.pmax, nullptr, true) : a.warp_smem;
     int per_warp = 1;
     const bool spawn = has_spawn_options(a);
-    if (small && multi && !spawn && a.npad_max <= kQuadMaxCells && 4 * wcap * ws_narrow <= 227 * 1024)
+    if (small && multi && !spawn && a.npad_max <= kQuadMaxCells && 4 * wcap * a.warp_smem <= 227 * 1024)
         per_warp = 4;
-    else if (small && a.npad_max <= kPairMaxCells && 2 * wcap * ws_narrow <= 227 * 1024)
+    else if (small && a.npad_max <= kPairMaxCells && 2 * wcap * a.warp_smem <= 227 * 1024)
         per_warp = 2;
-    if (per_warp == 1) return launch_groups(a, 32, multi, spawn, warps_per_cta, max_ctas, sms, st);
-    KArgs n = a;
-    n.warp_smem = ws_narrow;
-    return launch_groups(n, 32 / per_warp, multi, spawn, warps_per_cta, max_ctas, sms, st);
+    return launch_groups(a, 32 / per_warp, multi, spawn, warps_per_cta, max_ctas, sms, st);
 }
 
 int launch_copy(const void* src, void* dst, size_t n16, int blocks, void* stream) {
