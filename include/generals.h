@@ -444,7 +444,8 @@ int gen_sample_actions(gen_env *env, const float *d_logits, uint64_t seed, int32
  * wherever the games allow it -- at most two players, boards of at most
  * 1,024 padded cells (576 for four, without spawn options); 0 (default) = as 2 for
  * launches of at least 12 x the SM count games (24 x in multi-frame
- * launches), else 1.  GEN_ERR_BAD_ARG for NULL env or a mode outside 0..2. */
+ * launches), else 1, and for steps of small batches (up to 9 x the SM count
+ * games, more when they fall in several size buckets) a CTA per game.  GEN_ERR_BAD_ARG for NULL env or a mode outside 0..2. */
 int gen_set_lane_groups(gen_env *env, int mode);
 
 /* Tuning call, no counterpart in the paper (Section IV-G runs every board
@@ -454,7 +455,9 @@ int gen_set_lane_groups(gen_env *env, int mode);
  * work-list launch per frame (per rollout in the resident form): CTAs take
  * items -- up to a CTA's worth of one bucket's games, largest boards first --
  * from an atomic counter and carve their shared memory per item; 0 (default)
- * = 2 for batches of more than four buckets, else 1.  The work list's
+ * = one launch of a CTA per game for small batches (up to 27 x the SM count
+ * games, 40 x in four buckets or fewer), else 2 for batches of more than four
+ * buckets, else 1.  The work list's
  * counter belongs to the environment: order its calls on one stream.
  * GEN_ERR_BAD_ARG for NULL env or a form outside 0..2. */
 int gen_set_batch_form(gen_env *env, int form);

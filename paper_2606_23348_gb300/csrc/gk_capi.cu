@@ -282,8 +282,9 @@ int launch_one(const Bucket& b, const KArgs& a, void* stream, const char* what) 
     return GEN_OK;
 }
 
-// Every game, one launch per size bucket; buckets after the first run on
-// side streams forked from and joined back into `stream`.
+// Every game, in one launch by a CTA per game for small batches, else one
+// launch per size bucket (buckets after the first run on side streams forked
+// from and joined back into `stream`) or one work-list launch.
 // The work-list form serves batches of several buckets.  By default it takes
 // batches of more than four buckets: there the per-bucket launches are many
 // and small (mixed 32,768 games, 15 buckets: 136 against 131 M frames/s per
@@ -298,6 +299,15 @@ bool use_worklist(const gen_env* e) {
 template <class Fill>
 int launch_buckets(gen_env* e, int op, Fill fill, void* stream, const char* what) {
     const size_t nb = e->buckets.size();
+    if (nb > 1 && e->batch_form == 0) {
+        KArgs a = base_args(e, e->all, op);
+        a.list = e->d_order;  // largest boards first
+        fill(a);
+        bool taken = false;
+        const int rc = gk::launch_small(a, (int)nb, stream, &taken);
+        if (rc != 0) return cuda_fail((cudaError_t)rc, what);
+        if (taken) return GEN_OK;
+    }
     if (use_worklist(e)) {
         KArgs a = base_args(e, e->all, op);
         fill(a);
@@ -1554,7 +1564,7 @@ static int tune_env_forms(gen_env* e, int steps, int sms, std::string& rep) {
     if (rc == GEN_OK && t->buckets.size() > 1) {
         float bt = 1e30f;
         rep += "batch:";
-        for (int bf : {1, 2}) {
+        for (int bf : {0, 1, 2}) {
             t->batch_form = bf;
             const float ms = time_calls(step, steps, s, a, b);
             snprintf(line, sizeof(line), " %d=%.4fms", bf, ms);

@@ -780,6 +780,60 @@ __device__ int resolve_move(const Game& g, const Smem& s, int p, int32_t act, ui
     return 0;
 }
 
+// ---- the players' moves of one turn (Sec. IV-D, IV-E) ------------------------
+// In rotating priority, each checked when it runs (Q1).  my_act: lane p's is
+// player p's.  alive and eliminated end up the same on every lane; invalid
+// and sat count on lane 0.
+template <int LW>
+__device__ __forceinline__ void play_moves(const Game& g, const Smem& s, const Grp<LW>& t, uint32_t turn, int32_t my_act,
+                                           uint32_t& alive, uint32_t& eliminated, uint32_t& invalid, uint32_t& sat) {
+    int p = (int)(turn % (uint32_t)g.P);
+    for (int k = 0; k < g.P; ++k, p = p + 1 == g.P ? 0 : p + 1) {
+        const int32_t act = t.shfl(my_act, p);
+        int cap = 0;
+        if (t.lane == 0 && ((alive >> p) & 1u)) cap = resolve_move(g, s, p, act, alive, invalid, sat);
+        cap = t.shfl(cap, 0);
+        alive = t.shfl(alive, 0);
+        t.sync();
+        if (cap) {
+            // land transfer: every other cell of the loser, army - army/2 (Q7)
+            const int dst = cap & 0xFFFF, q = (cap >> 16) - 1;
+            eliminated |= 1u << q;
+            for (int c = t.lane; c < g.N; c += LW) {
+                if (c != dst && s.owner[c] == q) {
+                    s.owner[c] = (int8_t)p;
+                    const int av = s.army[c];
+                    s.army[c] = (int16_t)(av - (av >> 1));
+                }
+            }
+            t.sync();
+        }
+    }
+}
+
+// ---- termination and reward (Sec. III, IV-D, IV-E; Q17, Q21) -------------------
+// Returns the done code; lane p's reward is player p's.
+__device__ __forceinline__ uint32_t outcome(const KArgs& a, const Game& g, int lane, uint32_t turn, uint32_t alive,
+                                            uint32_t eliminated, float& reward) {
+    uint32_t done = 0;
+    if (g.mode == 1) {
+        const bool dead0 = (alive & 0x3u) == 0u, dead1 = (alive & 0xCu) == 0u;
+        if (dead0 || dead1) {
+            done = 1;
+            const bool mine_dead = ((lane >> 1) == 0) ? dead0 : dead1;
+            reward = mine_dead ? -1.0f : 1.0f;
+        }
+    } else {
+        if ((eliminated >> lane) & 1u) reward = -1.0f;
+        if (__popc(alive) <= 1) {
+            done = 1;
+            if ((alive >> lane) & 1u) reward = 1.0f;
+        }
+    }
+    if (!done && a.max_turns > 0 && turn >= (uint32_t)a.max_turns) done = 2;
+    return done;
+}
+
 // ---- growth + bitsets + army totals, 16 cells per lane ---------------------
 // Bytes are handled four at a time inside 32-bit words.  Per-cell flags are
 // bytes of 0 or 1 (or 0x80); dot products do the rest: four flags times powers
@@ -1143,17 +1197,19 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x, const Grp<LW>& t)
 // 4 x 4096 legal pairs); lane p then walks the chunks of the lane holding
 // player p's pair and selects the bit by popcount bisection, every player at
 // once.
+// u: on lanes 2p and 2p + 1 player p's two draws (policy_draws).
 // Returns, on lane p < P, player p's action; DIRECT also stores it.
+__device__ __forceinline__ uint32_t policy_draws(const KArgs& a, const Game& g, uint32_t frame, uint64_t gid, int lane) {
+    if (lane >= 2 * g.P) return 0u;
+    return hdraw(hkey(a.policy_seed, gid, frame, (uint64_t)(lane >> 1)), (uint64_t)(lane & 1));
+}
 template <bool DIRECT, int LW>
-__device__ int32_t policy_pass(const KArgs& a, const Game& g, const Smem& s, uint32_t alive, bool finished,
-                               uint32_t frame, uint64_t gid, const Grp<LW>& t) {
+__device__ int32_t policy_pass(const KArgs& a, const Game& g, const Smem& s, uint32_t alive, bool finished, uint32_t u,
+                               const Grp<LW>& t) {
     const int nch = g.nch;
     const int cpl = (nch + LW - 1) / LW;  // consecutive chunks per lane
     const int c_lo = t.lane * cpl;
     const int c_hi = min(c_lo + cpl, nch);
-    // lanes 2p and 2p + 1 hash player p's two draws
-    uint32_t u = 0;
-    if (t.lane < 2 * g.P) u = hdraw(hkey(a.policy_seed, gid, frame, (uint64_t)(t.lane >> 1)), (uint64_t)(t.lane & 1));
     int my_lane = -1;     // the lane whose chunks hold this lane's player's pair
     uint32_t my_rank = 0;  // the pair's index among that lane's
     bool my_half = false;
@@ -1329,7 +1385,8 @@ __device__ __forceinline__ void finish_frame(const KArgs& a, const Game& g, cons
     } else if (a.next_actions) {
         output_pass<false, true>(a, g, s, alive, fin, t, 0);
     }
-    if (a.next_actions) my_act = policy_pass<!MULTI, LW>(a, g, s, alive, fin, frame, game_id_of<UNI>(a, gidx), t);
+    if (a.next_actions)
+        my_act = policy_pass<!MULTI, LW>(a, g, s, alive, fin, policy_draws(a, g, frame, game_id_of<UNI>(a, gidx), t.lane), t);
 }
 
 __device__ __forceinline__ void store_scalars(const KArgs& a, int gidx, uint32_t turn, uint32_t frame, uint32_t epoch,
@@ -1427,51 +1484,13 @@ __device__ __forceinline__ void run_game(const KArgs& a, const Smem& s, char* wa
         if (a.op == OP_STEP && !finished) {
             if (MULTI && a.action_log && t.lane < g.P)
                 a.action_log[(int64_t)f * a.slot_stride + g.player_off + t.lane] = my_act;
-            // moves in rotating priority, each checked when it runs (Q1)
-            uint32_t eliminated = 0;
-            uint32_t inv0 = 0, sat0 = 0;
-            for (int k = 0; k < g.P; ++k) {
-                const int p = (int)((turn + (uint32_t)k) % (uint32_t)g.P);
-                const int32_t act = t.shfl(my_act, p);
-                int cap = 0;
-                if (t.lane == 0 && ((alive >> p) & 1u)) cap = resolve_move(g, s, p, act, alive, inv0, sat0);
-                cap = t.shfl(cap, 0);
-                alive = t.shfl(alive, 0);
-                t.sync();
-                if (cap) {
-                    // land transfer: every other cell of the loser, army - army/2 (Q7)
-                    const int dst = cap & 0xFFFF, q = (cap >> 16) - 1;
-                    eliminated |= 1u << q;
-                    for (int c = t.lane; c < g.N; c += LW) {
-                        if (c != dst && s.owner[c] == q) {
-                            s.owner[c] = (int8_t)p;
-                            const int av = s.army[c];
-                            s.army[c] = (int16_t)(av - (av >> 1));
-                        }
-                    }
-                    t.sync();
-                }
-            }
+            uint32_t eliminated = 0, inv0 = 0, sat0 = 0;
+            play_moves(g, s, t, turn, my_act, alive, eliminated, inv0, sat0);
             invalid += t.shfl(inv0, 0);
             saturated += t.shfl(sat0, 0);
             turn += 1;
             saturated += cell_pass<IN_TURN>(g, s, (turn % 2u) == 0u, (turn % 50u) == 0u, t);
-            // termination and reward (Sec. III, IV-D, IV-E; Q17, Q21)
-            if (g.mode == 1) {
-                const bool dead0 = (alive & 0x3u) == 0u, dead1 = (alive & 0xCu) == 0u;
-                if (dead0 || dead1) {
-                    done = 1;
-                    const bool mine_dead = ((t.lane >> 1) == 0) ? dead0 : dead1;
-                    my_reward = mine_dead ? -1.0f : 1.0f;
-                }
-            } else {
-                if ((eliminated >> t.lane) & 1u) my_reward = -1.0f;
-                if (__popc(alive) <= 1) {
-                    done = 1;
-                    if ((alive >> t.lane) & 1u) my_reward = 1.0f;
-                }
-            }
-            if (!done && a.max_turns > 0 && turn >= (uint32_t)a.max_turns) done = 2;
+            done = outcome(a, g, t.lane, turn, alive, eliminated, my_reward);
             if (done) {
                 if (a.auto_reset) {
                     epoch += 1;

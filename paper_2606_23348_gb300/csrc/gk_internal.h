@@ -91,7 +91,7 @@ struct KArgs {
     int32_t spawn_dmax;     // cap on a general's distance to every earlier one (0: none)
     int32_t spawn_bfs;      // 1: spacing in BFS steps around mountains
     int32_t castle_radius;  // > 0: a neutral castle within this many steps of every general
-    // games per warp: 0 by batch size, 1 a warp per game, 2 two or four per
+    // games per warp: 0 by batch size (a CTA per game for small ones), 1 a warp per game, 2 two or four per
     // warp whenever the games allow (two players, small boards)
     int32_t lane_groups;
 };
@@ -238,6 +238,10 @@ int launch_worklist(const KArgs& a, const WArgs& w, int cta_smem, int ctas, void
 // Launch the step kernel with `warps_per_cta` games per CTA on `stream`.
 // Returns a cudaError_t value.
 int launch_step(const KArgs& a, int warps_per_cta, int max_ctas, void* stream);
+
+// A step over games of several size classes by a CTA per game, if the batch is
+// small enough for that to be the faster form (*taken).  Returns a cudaError_t.
+int launch_small(const KArgs& a, int classes, void* stream, bool* taken);
 
 // Fill the device's constant tables (board column masks); once per device,
 // synchronous.  Returns a cudaError_t value.

@@ -15,6 +15,8 @@ StepKernel rollout_kernel(int lw, bool uniform, bool spawn);
 int fill_rollout_columns();
 WorklistKernel worklist_kernel(bool multi, bool spawn);
 int fill_worklist_columns();
+int launch_team(const KArgs& a, int sms, void* stream);
+int fill_team_columns();
 
 __global__ void k_copy(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t n) {
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -130,7 +132,7 @@ int init_tables() {
     if (e != cudaSuccess) return (int)e;
     std::lock_guard<std::mutex> lk(mu);
     if (dev >= 0 && dev < 64 && ready[dev]) return 0;
-    for (int (*fill)() : {fill_columns, fill_rollout_columns, fill_worklist_columns}) {
+    for (int (*fill)() : {fill_columns, fill_rollout_columns, fill_worklist_columns, fill_team_columns}) {
         const int f = fill();
         if (f != 0) return f;
     }
@@ -198,6 +200,42 @@ int launch_groups(const KArgs& a, int lw, bool multi, bool spawn, int fixed_warp
     return launch_chained(f, dim3(blocks), dim3(32 * warps), smem, st, a);
 }
 
+// SMs of the first device used: only launch shapes depend on it
+int sm_count() {
+    static std::atomic<int> count{0};
+    int sms = count.load(std::memory_order_relaxed);
+    if (sms == 0) {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        sms = n > 0 ? n : 1;
+        count.store(sms, std::memory_order_relaxed);
+    }
+    return sms;
+}
+
+// A CTA per game (gk_team.cu) while the batch is small.  Of one size class, up
+// to 9 games per SM, where three warps per game still run all at once: 32
+// frames of 24x24 1v1 games, against a warp per game, 85 / 122 / 162 us for
+// 64 / 1,024 / 1,400 games against 127 / 142 / 184, but 188 against 185 for
+// 1,536.
+constexpr int kTeamGames = 9;
+// Of several classes, against one launch per class on forked streams (up to
+// four classes; 1v1 games of 15..30 a side, per frame: 1,024 games 8.4
+// against 21.1 us, 6,144 23.9 against 29.4, 8,192 31.0 against 32.2, 12,288
+// 46.9 against 39.4) or against the work list (mixed games of 20..40 a side:
+// 512 games 12.9 against 21.4 us, 4,096 37.7 against 43.0, 6,144 51.7 against
+// 46.8).
+constexpr int kTeamGamesFewClasses = 40, kTeamGamesManyClasses = 27;
+bool team_batch(const KArgs& a, int per_sm, int sms) {
+    return a.op == OP_STEP && a.do_outputs && a.lane_groups == 0 && a.n_items <= per_sm * sms;
+}
+int launch_small(const KArgs& a, int classes, void* stream, bool* taken) {
+    const int sms = sm_count();
+    *taken = team_batch(a, classes > 4 ? kTeamGamesManyClasses : kTeamGamesFewClasses, sms);
+    return *taken ? launch_team(a, sms, stream) : 0;
+}
+
 int launch_step(const KArgs& a, int warps_per_cta, int max_ctas, void* stream) {
     if (a.n_items <= 0) return 0;
 
@@ -207,17 +245,10 @@ int launch_step(const KArgs& a, int warps_per_cta, int max_ctas, void* stream) {
         const int e = allow_max_smem();
         if (e != 0) return e;
     }
-    static std::atomic<int> sm_count{0};  // of the first device used: only the launch shape depends on it
-    int sms = sm_count.load(std::memory_order_relaxed);
-    if (sms == 0) {
-        int dev = 0, n = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        sms = n > 0 ? n : 1;
-        sm_count.store(sms, std::memory_order_relaxed);
-    }
-    // several games per warp for small two-player boards, once the batch is large enough: below it a warp per game is
-    // faster (measured on 24x24 1v1: 1,024 games per frame 98 against 87 M
+    const int sms = sm_count();
+    if (team_batch(a, kTeamGames, sms)) return launch_team(a, sms, stream);
+    // several games per warp for small two-player boards, once the batch is
+    // large enough: below it a warp per game is faster (measured on 24x24 1v1: 1,024 games per frame 98 against 87 M
     // frames/s, resident 194 against 122 M; pairs win from 2,048 games per
     // frame and 4,096 resident)
     const bool large = a.n_items >= (multi ? 24 : 12) * sms;

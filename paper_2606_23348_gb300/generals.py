@@ -357,7 +357,7 @@ class GeneralsEnv:
     def set_lane_groups(self, mode: int):
         """Games per warp in the step kernels: LANES_WARP (one), LANES_NARROW
         (two, four in rollouts, wherever the games allow) or LANES_AUTO (by
-        batch size)."""
+        batch size; a CTA per game for small ones)."""
         _check(self.lib.gen_set_lane_groups(self.h, int(mode)), "gen_set_lane_groups")
 
     BATCH_AUTO, BATCH_BUCKETS, BATCH_WORKLIST = 0, 1, 2
@@ -365,7 +365,8 @@ class GeneralsEnv:
     def set_batch_form(self, form: int):
         """How a batch of several size buckets launches: BATCH_BUCKETS (one
         launch per bucket), BATCH_WORKLIST (one persistent work-list launch)
-        or BATCH_AUTO (the work list for batches of more than four buckets)."""
+        or BATCH_AUTO (one launch of a CTA per game for small batches, the work
+        list for larger ones of more than four buckets)."""
         _check(self.lib.gen_set_batch_form(self.h, int(form)), "gen_set_batch_form")
 
     def set_sample_form(self, form: int):

@@ -297,6 +297,19 @@ def test_generator_rows_at_word_edges(H, W, mode, P, lanes):
     rollout_policy(env, orc, 16, policy_seed=3, check_every=1, tag=f"{H}x{W}")
 
 
+@pytest.mark.parametrize("auto_reset", [0, 1])
+@pytest.mark.parametrize("H,W,mode,P", [(1, 2, 0, 2), (40, 1, 2, 3), (7, 9, 1, 4), (16, 16, 0, 2), (5, 33, 2, 2),
+                                        (31, 17, 2, 8), (64, 64, 2, 8)])
+def test_cta_per_game_edges(H, W, mode, P, auto_reset):
+    """A CTA per game (small batches, the default there): boards of one chunk
+    or an odd number, rows wider than a word, two to eight warps a game,
+    truncation with a new map and with a frozen game."""
+    full = lambda x: np.full(5, x, np.int32)  # noqa: E731
+    env, orc = pair(full(H), full(W), full(mode), full(P), seed=31, n_cities=1, min_general_dist=1, max_turns=11,
+                    auto_reset=auto_reset)
+    rollout_policy(env, orc, 24, policy_seed=6, check_every=1, tag=f"{H}x{W}")
+
+
 def test_spawn_range_curriculum_update():
     import torch
     G = 48
