@@ -524,19 +524,16 @@ int gen_features_build(gen_features *f, float *d_out, void *stream);
  * builder created without a window. */
 int gen_features_build_ex(gen_features *f, float *d_out, int32_t *d_series, void *stream);
 
-/* Tuning call, no counterpart in the paper.  Times `steps` builds in each
- * form (gen_features_set_form 1 and 2) into d_out and keeps the faster;
- * *form_out (may be NULL) receives it.  The first build folds the current
- * frame; the timed ones repeat it (a repeated build in one frame changes
- * nothing), so d_out holds this frame's features afterwards.  Synchronous. */
+/* Tuning call, no counterpart in the paper; kept for its callers.  It chose
+ * between two ways to spread a game over the GPU; one CTA per (game, player)
+ * is now the fastest at every batch size and always runs.  Folds the current
+ * frame into d_out as gen_features_build does; *form_out (may be NULL)
+ * receives 2.  GEN_ERR_BAD_ARG for NULL pointers or steps < 1.  Synchronous. */
 int gen_features_autotune(gen_features *f, float *d_out, int steps, int *form_out);
 
-/* Tuning call, no counterpart in the paper.  How the builder spreads a
- * game over the GPU (the bytes written are the same): 1 = one warp per
- * game, players in turn; 2 = one CTA per (game, player), its warps sharing
- * the player's 128-cell chunks, for batches too small to fill the GPU one
- * warp per game; 0 (default) = 2 while games x the most players per game is
- * at most 56 x the SM count, else 1.  GEN_ERR_BAD_ARG outside 0..2. */
+/* Tuning call, no counterpart in the paper; kept for its callers.  The form
+ * (0..2) changes nothing, see gen_features_autotune.  GEN_ERR_BAD_ARG outside
+ * 0..2. */
 int gen_features_set_form(gen_features *f, int form);
 
 /* Free a builder's memory (App. A feature memory). */

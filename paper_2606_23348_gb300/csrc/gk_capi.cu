@@ -1276,7 +1276,6 @@ struct gen_features {
     gen_env* env = nullptr;
     int hist = 0;
     int window = 0;
-    int form = 0;  // 0 by batch size, 1 one warp per game, 2 one CTA per game
     void* d_mem = nullptr;  // one allocation: headers, masks, last army, last turn, ring
     gk::FArgs args{};
 };
@@ -1313,6 +1312,8 @@ int gen_features_create_ex(gen_features** out, gen_env* e, int hist, int window)
     }
     f->d_mem = m;
     gk::FArgs& a = f->args;
+    a.npad_mean = (int32_t)(e->plane_cells / e->player_slots);
+    a.n_players = e->player_slots;
     a.info = e->d_info;
     a.army = e->d_army;
     a.owner = e->d_owner;
@@ -1330,6 +1331,10 @@ int gen_features_create_ex(gen_features** out, gen_env* e, int hist, int window)
     a.window = window;
     a.series_ring = window > 0 ? reinterpret_cast<int2*>(m + hdr + bits + army + turn + ring) : nullptr;
     a.series_out = nullptr;
+    if (e->uniform) {
+        a.uniform = 1;
+        a.ushape = e->h_info[0];
+    }
     *out = f;
     return GEN_OK;
 }
@@ -1361,7 +1366,7 @@ int gen_features_build_ex(gen_features* f, float* d_out, int32_t* d_series, void
     gk::FArgs a = f->args;
     a.out = d_out;
     a.series_out = reinterpret_cast<int2*>(d_series);
-    const int rc = gk::launch_features(a, f->env->pmax, f->form, stream);
+    const int rc = gk::launch_features(a, f->env->pmax, stream);
     if (rc != 0) return cuda_fail((cudaError_t)rc, "feature launch");
     return GEN_OK;
 }
@@ -1369,39 +1374,21 @@ int gen_features_build_ex(gen_features* f, float* d_out, int32_t* d_series, void
 int gen_features_autotune(gen_features* f, float* d_out, int steps, int* form_out) {
     if (!f || !d_out) return fail(GEN_ERR_BAD_ARG, "NULL argument");
     if (steps < 1) return fail(GEN_ERR_BAD_ARG, "steps < 1");
+    // one form is the fastest at every size: this frame's build, and its number
     cudaStream_t s = nullptr;
-    cudaEvent_t a = nullptr, b = nullptr;
     CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking), "autotune stream");
-    cudaEventCreate(&a);
-    cudaEventCreate(&b);
-    // the first build folds the current frame; the timed ones repeat it, so
-    // both forms do the same work and the memory is as one build leaves it
     int rc = gen_features_build_ex(f, d_out, nullptr, s);
-    float best = 1e30f;
-    int best_form = f->form;
-    for (int form : {1, 2}) {
-        if (rc) break;
-        f->form = form;
-        auto build = [&]() { return gen_features_build_ex(f, d_out, nullptr, s); };
-        const float ms = time_calls(build, steps, s, a, b);
-        if (ms < best) {
-            best = ms;
-            best_form = form;
-        }
-    }
-    cudaEventDestroy(a);
-    cudaEventDestroy(b);
+    const cudaError_t ce = cudaStreamSynchronize(s);
     cudaStreamDestroy(s);
-    f->form = best_form;
+    if (rc == GEN_OK && ce != cudaSuccess) rc = cuda_fail(ce, "feature build");
     if (rc) return rc;
-    if (form_out) *form_out = best_form;
+    if (form_out) *form_out = 2;
     return GEN_OK;
 }
 
 int gen_features_set_form(gen_features* f, int form) {
     if (!f) return fail(GEN_ERR_BAD_ARG, "features is NULL");
     if (form < 0 || form > 2) return fail(GEN_ERR_BAD_ARG, "form %d outside [0, 2]", form);
-    f->form = form;
     return GEN_OK;
 }
 

@@ -14,19 +14,19 @@
 // 0 when visible or never seen; coordinates col / (W - 1), row / (H - 1);
 // frames before the episode count as zero planes.
 //
-// Two forms of the same computation.  k_features: one warp per game -- the
-// board is staged in shared memory once, then each player in turn gets a
-// visibility bitset (3x3 dilation of its team's cells) and a pass over the
-// cells, four consecutive cells per lane, that reads the memory, writes the
-// 24 + 2K channels with 16-byte streaming stores and writes the folded memory
-// back.  k_features_cta, for batches too small to fill the GPU one warp per
-// game: one CTA per (game, player); each warp stages the memory and history
-// planes of two of the player's 128-cell chunks with cp.async while one warp
-// builds the player's bitset and others the scoreboard, then writes those
-// chunks; the player's memory header is read before the CTA's last barrier
-// and written after it.
+// One CTA per (game, player), its warps sharing the player's 128-cell chunks:
+// each warp stages the memory and history planes of its chunks with cp.async
+// while one warp builds the player's visibility bitset (3x3 dilation of its
+// team's cells) and others the scoreboard, then writes the chunks' 24 + 2K
+// rows with 16-byte streaming stores, four consecutive cells per lane; the
+// player's memory header is read before the CTA's last barrier and written
+// after it.
 // HBM-bound: per player and cell it moves 4 (24 + 2K) bytes of output,
-// 2 * 2K bytes of history and 15 bytes of memory.
+// 2 * 2K bytes of history and 15 bytes of memory.  Step and build of 16,384
+// 24x24 1v1 games 627 us with a chunk per warp, 702 us with two, 707 us by a
+// warp per game with the players in turn and 681 us by a warp per player
+// (both wait for the loads of each chunk in turn); 65,536 games 2,499 against
+// 2,613 us, 1,000 30x30 free-for-all games 255 against 319 us.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -40,14 +40,6 @@ namespace gk {
 namespace {
 
 constexpr unsigned kAll = 0xFFFFFFFFu;
-constexpr int kWarps = 8;
-
-// shared memory of one warp: board (4 bytes per cell), team and visibility
-// bitsets, scoreboard; a multiple of 16 bytes
-__host__ __device__ __forceinline__ int warp_bytes(int npad_max) {
-    const int nw_max = (npad_max + 31) >> 5;
-    return (4 * npad_max + 8 * nw_max + 64 + 8 * kMaxSide + 15) & ~15;
-}
 
 // the coordinate rows' values (Q32) by column and by row: column / (W - 1)
 // and row / (H - 1), 0 when the side is 1; computed once per game
@@ -159,6 +151,17 @@ __device__ __forceinline__ float4 f4_16(uint2 x) {
 __device__ __noinline__ float age_log(int dt) { return (float)(log(1.0 + (double)dt) / 5.0); }
 __device__ __forceinline__ float age_value(int dt) { return dt > 0 ? age_log(dt) : 0.0f; }
 
+// a game's description; of a uniform batch without a load, since the loads
+// that follow would wait for it
+__device__ __forceinline__ GameInfo feature_game(const FArgs& f, int gidx) {
+    if (!f.uniform) return f.info[gidx];
+    GameInfo gi = f.ushape;
+    gi.cell_off = gidx * gi.Npad;
+    gi.player_off = gidx * gi.P;
+    gi.plane_off = (int64_t)gidx * gi.P * gi.Npad;
+    return gi;
+}
+
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
                  "l"(gmem)
@@ -226,11 +229,9 @@ struct PlayerFrame {
     int nvalid;       // ring slots holding frames of this episode
 };
 
-// LOAD_HDR: the player's memory header is read from global memory here (the
-// warp form), else `h` holds it (the CTA form stages the headers)
-template <bool LOAD_HDR>
-__device__ __forceinline__ PlayerFrame player_frame_t(const FArgs& f, const GameInfo& gi, const GameScalars& sc,
-                                                      const int32_t* s_score, int p, int R, uint4 h) {
+// h: the player's memory header
+__device__ __forceinline__ PlayerFrame player_frame(const GameInfo& gi, const GameScalars& sc, const int32_t* s_score,
+                                                    int p, int R, uint4 h) {
     PlayerFrame x;
     x.p = p;
     x.tp = gi.mode == 1 ? (p >> 1) : p;
@@ -249,7 +250,6 @@ __device__ __forceinline__ PlayerFrame player_frame_t(const FArgs& f, const Game
     x.f_opp_land = (float)opp_land;
     x.f_opp_army = (float)opp_army;
     // memory header: clear on a new epoch, fold once per frame
-    if (LOAD_HDR) h = f.hdr[x.slot];
     x.cleared = h.x != sc.epoch + 1u;
     x.fold = x.cleared || h.y != sc.frame;
     x.n_fold = (x.cleared ? 0u : h.z) + (x.fold ? 1u : 0u);
@@ -283,8 +283,7 @@ __device__ __forceinline__ void player_tokens(const FArgs& f, const PlayerFrame&
 // cells c .. c+3 of one player: read and fold the memory, write the 24 + 2K
 // rows.  mem(mb, lea, let) supplies the memory of the four cells (zeros when
 // cleared) and ring_pair(back, own, enemy) the army planes `back` frames ago
-// (zeros where the episode has none): global loads for the warp form, a
-// shared-memory staging for the CTA form.
+// (zeros where the episode has none).
 template <class Mem, class Ring>
 __device__ __forceinline__ void cell_quad_from(const FArgs& f, const GameInfo& gi, const PlayerFrame& x, int turn,
                                                float f_turn, float f_phase, const int16_t* s_army,
@@ -410,95 +409,10 @@ __device__ __forceinline__ void cell_quad_from(const FArgs& f, const GameInfo& g
     }
 }
 
-// the warp form's cells: memory and ring planes loaded from global memory
-__device__ __forceinline__ void cell_quad(const FArgs& f, const GameInfo& gi, const PlayerFrame& x, int turn,
-                                          float f_turn, float f_phase, const int16_t* s_army, const int8_t* s_owner,
-                                          const int8_t* s_terrain, const uint32_t* s_vis, const float* s_coord,
-                                          int c) {
-    const int R = f.hist + 1;
-    const int64_t pc = gi.plane_off + (int64_t)x.p * gi.Npad + c;
-    auto mem = [&](uint32_t& mb, uint2& lea, int4& let) {
-        if (!x.cleared) {
-            mb = __ldcs(reinterpret_cast<const unsigned int*>(f.mem_bits + pc));
-            lea = __ldcs(reinterpret_cast<const uint2*>(f.mem_army + pc));
-            let = __ldcs(reinterpret_cast<const int4*>(f.mem_turn + pc));
-        }
-    };
-    auto ring_pair = [&](int back, uint2& o, uint2& e) {  // own / enemy planes `back` frames ago
-        o = make_uint2(0u, 0u);
-        e = o;
-        if (back < x.nvalid) {
-            const int sl = (x.head - back + R) % R;
-            o = __ldcs(reinterpret_cast<const uint2*>(f.ring + (int64_t)(2 * sl) * f.plane_cells + pc));
-            e = __ldcs(reinterpret_cast<const uint2*>(f.ring + (int64_t)(2 * sl + 1) * f.plane_cells + pc));
-        }
-    };
-    cell_quad_from(f, gi, x, turn, f_turn, f_phase, s_army, s_owner, s_terrain, s_vis, s_coord, c, mem, ring_pair);
-}
-
-__global__ void __launch_bounds__(256, 4) k_features(const FArgs f) {
-    chain_entry();
-    extern __shared__ __align__(16) char smem[];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int gidx = blockIdx.x * kWarps + wid;
-    if (gidx >= f.n_games) return;
-
-    const int nw_max = (f.npad_max + 31) >> 5;
-    char* base = smem + (size_t)wid * warp_bytes(f.npad_max);
-    int16_t* s_army = reinterpret_cast<int16_t*>(base);
-    int8_t* s_owner = reinterpret_cast<int8_t*>(base + 2 * f.npad_max);
-    int8_t* s_terrain = reinterpret_cast<int8_t*>(base + 3 * f.npad_max);
-    uint32_t* s_team = reinterpret_cast<uint32_t*>(base + 4 * f.npad_max);
-    uint32_t* s_vis = s_team + nw_max;
-    int32_t* s_score = reinterpret_cast<int32_t*>(s_vis + nw_max);  // land[8], army[8]
-    float* s_coord = reinterpret_cast<float*>(s_score + 16);         // [2 * kMaxSide]
-
-    const GameInfo gi = f.info[gidx];
-    const int N = gi.N, Npad = gi.Npad, P = gi.P;
-    const int nw = (Npad + 31) >> 5;
-    const GameScalars sc = f.scal[gidx];
-    const int R = f.hist + 1;
-
-    // board to shared memory, 16 bytes per lane and copy
-    {
-        const uint4* ga = reinterpret_cast<const uint4*>(f.army + gi.cell_off);
-        const uint4* go = reinterpret_cast<const uint4*>(f.owner + gi.cell_off);
-        const uint4* gt = reinterpret_cast<const uint4*>(f.terrain + gi.cell_off);
-        const int n16 = Npad >> 4;
-        for (int v = lane; v < 2 * n16; v += 32) reinterpret_cast<uint4*>(s_army)[v] = __ldg(ga + v);
-        for (int v = lane; v < n16; v += 32) {
-            reinterpret_cast<uint4*>(s_owner)[v] = __ldg(go + v);
-            reinterpret_cast<uint4*>(s_terrain)[v] = __ldg(gt + v);
-        }
-    }
-    coord_table(s_coord, gi.H, gi.W, lane, 32);
-    __syncwarp();
-
-    // public scoreboard (Sec. IV-B): land and army per player
-    for (int q = 0; q < P; ++q) score_of(s_army, s_owner, N, q, s_score, lane);
-    __syncwarp();
-
-    const int turn = (int)sc.turn;
-    const float f_turn = (float)turn;
-    const float f_phase = (float)(turn % 50) / 50.0f;
-
-    for (int p = 0; p < P; ++p) {
-        const int tp = gi.mode == 1 ? (p >> 1) : p;
-        vis_of(s_owner, s_team, s_vis, N, gi.W, nw, gi.mode, tp, (sc.alive >> p) & 1u, lane);
-        const PlayerFrame x = player_frame_t<true>(f, gi, sc, s_score, p, R, make_uint4(0u, 0u, 0u, 0u));
-        if (f.window > 0) player_tokens(f, x, lane == 0, (uint32_t)lane, 32u);
-        for (int c = 4 * lane; c < Npad; c += 128)
-            cell_quad(f, gi, x, turn, f_turn, f_phase, s_army, s_owner, s_terrain, s_vis, s_coord, c);
-        if (x.fold && lane == 0) f.hdr[x.slot] = make_uint4(sc.epoch + 1u, sc.frame, x.n_fold, 0u);
-        __syncwarp();
-    }
-}
-
 // shared memory of the one-player CTA: board, the player's visibility bitset
 // and a scratch bitset, scoreboard, coordinate table, the player's memory
-// header, then per warp the staging of kItemsPerBatch items; a multiple of
+// header, then per warp the staging of its items; a multiple of
 // 16 bytes
-constexpr int kItemsPerBatch = 2;
 __host__ __device__ __forceinline__ int cta_hdr_offset(int npad_max) {  // 16-byte aligned
     const int nw_max = (npad_max + 31) >> 5;
     return (4 * npad_max + 8 * nw_max + 64 + 8 * kMaxSide + 15) & ~15;
@@ -508,8 +422,8 @@ __host__ __device__ __forceinline__ int cta_head_bytes(int npad_max) { return ct
 // turn (16 B) of the lane's four cells, then K (own, enemy) ring plane pairs
 // (8 + 8 B)
 __host__ __device__ __forceinline__ int item_stage_bytes(int hist) { return 32 * (28 + 16 * hist); }
-__host__ __device__ __forceinline__ int cta_bytes(int npad_max, int hist, int warps) {
-    return cta_head_bytes(npad_max) + warps * kItemsPerBatch * item_stage_bytes(hist);
+__host__ __device__ __forceinline__ int cta_bytes(int npad_max, int hist, int warps, int items) {
+    return cta_head_bytes(npad_max) + warps * items * item_stage_bytes(hist);
 }
 
 __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
@@ -553,18 +467,19 @@ __device__ __forceinline__ void stage_item(const FArgs& f, const HdrState& y, in
     }
 }
 
-// One CTA per (game, player): CTA b takes player b mod pmax of game
-// b / pmax (CTAs of absent players return at once).  The board and the
-// player's header are staged first; the items' memory and history planes are
-// in flight while one warp builds the player's visibility bitset and the
-// others the scoreboard (a warp per player); then warp w takes the player's
-// 128-cell chunks w, w + warps, ... kItemsPerBatch at a time.
-__global__ void __launch_bounds__(1024) k_features_cta(const FArgs f, int pmax) {
+// CTA b takes player b mod pmax of game b / pmax (CTAs of absent players
+// return at once).  The board and the player's header are staged first; the
+// chunks' memory and history planes are in flight while one warp builds the
+// player's visibility bitset and the others the scoreboard (a warp per
+// player); then warp w takes the player's 128-cell chunks w, w + warps, ...
+// ITEMS at a time.
+template <int ITEMS>
+__global__ void __launch_bounds__(1024) k_features(const FArgs f, int pmax) {
     extern __shared__ __align__(16) char smem[];
     chain_entry();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int gidx = blockIdx.x / pmax, p = blockIdx.x - gidx * pmax;
-    const GameInfo gi = f.info[gidx];
+    const GameInfo gi = feature_game(f, gidx);
     const int N = gi.N, Npad = gi.Npad, P = gi.P;
     if (p >= P) return;  // the same for the whole CTA
 
@@ -577,7 +492,7 @@ __global__ void __launch_bounds__(1024) k_features_cta(const FArgs f, int pmax) 
     int32_t* s_score = reinterpret_cast<int32_t*>(s_team + nw_max);         // land[8], army[8]
     float* s_coord = reinterpret_cast<float*>(s_score + 16);                // [2 * kMaxSide]
     uint4* s_hdr = reinterpret_cast<uint4*>(smem + cta_hdr_offset(f.npad_max));
-    char* s_stage = smem + cta_head_bytes(f.npad_max) + (size_t)wid * kItemsPerBatch * item_stage_bytes(f.hist);
+    char* s_stage = smem + cta_head_bytes(f.npad_max) + (size_t)wid * ITEMS * item_stage_bytes(f.hist);
 
     const int nw = (Npad + 31) >> 5;
     const GameScalars sc = f.scal[gidx];
@@ -606,10 +521,10 @@ __global__ void __launch_bounds__(1024) k_features_cta(const FArgs f, int pmax) 
     const uint4 h = *s_hdr;
     const HdrState y = hdr_state(h, sc, R);
     // this warp's chunks are wid, wid + nwarps, ...; batch b holds the
-    // kItemsPerBatch of them from the (b * kItemsPerBatch)-th on
+    // ITEMS of them from the (b * ITEMS)-th on
     auto stage_batch = [&](int b) {
-        for (int j = 0; j < kItemsPerBatch; ++j) {
-            const int k = wid + nwarps * (b * kItemsPerBatch + j), c = 128 * k + 4 * lane;
+        for (int j = 0; j < ITEMS; ++j) {
+            const int k = wid + nwarps * (b * ITEMS + j), c = 128 * k + 4 * lane;
             if (k >= chunks) break;
             if (c < Npad) stage_item(f, y, q0 + c, s_stage + j * item_stage_bytes(f.hist), lane);
         }
@@ -627,13 +542,13 @@ __global__ void __launch_bounds__(1024) k_features_cta(const FArgs f, int pmax) 
     const int turn = (int)sc.turn;
     const float f_turn = (float)turn;
     const float f_phase = (float)(turn % 50) / 50.0f;
-    const PlayerFrame x = player_frame_t<false>(f, gi, sc, s_score, p, R, h);
+    const PlayerFrame x = player_frame(gi, sc, s_score, p, R, h);
     const int mine = chunks > wid ? (chunks - wid + nwarps - 1) / nwarps : 0;
-    for (int b = 0; kItemsPerBatch * b < mine; ++b) {
+    for (int b = 0; ITEMS * b < mine; ++b) {
         if (b > 0) stage_batch(b);
         asm volatile("cp.async.wait_all;" ::: "memory");
-        for (int j = 0; j < kItemsPerBatch; ++j) {
-            const int k = wid + nwarps * (b * kItemsPerBatch + j);
+        for (int j = 0; j < ITEMS; ++j) {
+            const int k = wid + nwarps * (b * ITEMS + j);
             if (k >= chunks) break;
             // the player's tokens are shared by its first min(chunks, warps) chunks
             if (f.window > 0) {
@@ -671,7 +586,7 @@ __global__ void __launch_bounds__(1024) k_features_cta(const FArgs f, int pmax) 
 
 }  // namespace
 
-int launch_features(const FArgs& f, int pmax, int form, void* stream) {
+int launch_features(const FArgs& f, int pmax, void* stream) {
     if (f.n_games <= 0) return 0;
     static std::atomic<int> sm_count{0};  // of the first device used: only the launch shape depends on it
     int sms = sm_count.load(std::memory_order_relaxed);
@@ -682,33 +597,32 @@ int launch_features(const FArgs& f, int pmax, int form, void* stream) {
         sms = n > 0 ? n : 1;
         sm_count.store(sms, std::memory_order_relaxed);
     }
-    // the CTA form while the batch has at most 56 x the SM count players
-    // (measured on 24x24 1v1, each build the first of its frame: 512 games
-    // 28.5 against 69.3 us, 4,096 games 184.8 against 186.4 us, 8,192 games
-    // 360 against 335 us)
-    if (form == 0) form = (int64_t)f.n_games * pmax <= 56 * (int64_t)sms ? 2 : 1;
-    if (form == 2) {
-        // a CTA per (game, player) with a warp per kItemsPerBatch chunks, as
-        // many as the staging leaves room for in shared memory
-        const int chunks = (f.npad_max + 127) >> 7;
-        const int per_warp = kItemsPerBatch * item_stage_bytes(f.hist);
-        const int fit = (227 * 1024 - cta_head_bytes(f.npad_max)) / per_warp;
-        const int warps = std::max(1, std::min(std::min(32, fit), (chunks + kItemsPerBatch - 1) / kItemsPerBatch));
-        const int smem = cta_bytes(f.npad_max, f.hist, warps);
-        static SmemLimit limit;
-        const void* fn = (const void*)k_features_cta;
-        const int e = limit.raise(&fn, 1, smem);
-        if (e != 0) return e;
-        return launch_chained(k_features_cta, dim3((unsigned)((int64_t)f.n_games * pmax)), dim3(32 * warps), smem,
-                              (cudaStream_t)stream, f, pmax);
+    // Warps per player and chunks of 128 cells per warp at a time (32 warps of
+    // an SM run at once at 62 registers).  A batch that fits gets a warp per
+    // chunk of the largest board, or, where only that fits, a warp per two
+    // (512 24x24 1v1 games' self-play frame 37.2 against 39.5 us); larger ones
+    // a warp per chunk of the mean board, larger boards taking several rounds
+    // (2,048 mixed games of 20..40 a side 300 us, for the largest board 394).
+    const int stage = item_stage_bytes(f.hist);
+    const int fit = (227 * 1024 - cta_head_bytes(f.npad_max)) / stage;
+    const int largest = (f.npad_max + 127) >> 7, mean = (f.npad_mean + 127) >> 7;
+    const int64_t room = 32 * (int64_t)sms;
+    int warps = mean, items = 1;
+    if (f.n_players * (int64_t)largest <= room) {
+        warps = largest;
+    } else if (f.n_players * (int64_t)((largest + 1) / 2) <= room && 2 * ((largest + 1) / 2) <= fit) {
+        warps = (largest + 1) / 2;
+        items = 2;
     }
-    const int smem = kWarps * warp_bytes(f.npad_max);
+    warps = std::max(1, std::min(std::min(32, fit / items), warps));
+    const int smem = cta_bytes(f.npad_max, f.hist, warps, items);
+    void (*const fn)(FArgs, int) = items == 1 ? k_features<1> : k_features<2>;
     static SmemLimit limit;
-    const void* fn = (const void*)k_features;
-    const int e = limit.raise(&fn, 1, smem);
+    static const void* const fns[2] = {(const void*)k_features<1>, (const void*)k_features<2>};
+    const int e = limit.raise(fns, 2, smem);
     if (e != 0) return e;
-    const int blocks = (f.n_games + kWarps - 1) / kWarps;
-    return launch_chained(k_features, dim3(blocks), dim3(32 * kWarps), smem, (cudaStream_t)stream, f);
+    return launch_chained(fn, dim3((unsigned)((int64_t)f.n_games * pmax)), dim3(32 * warps), smem, (cudaStream_t)stream,
+                          f, pmax);
 }
 
 }  // namespace gk

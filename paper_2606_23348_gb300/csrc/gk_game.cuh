@@ -1110,8 +1110,8 @@ __device__ __forceinline__ uint64_t chunk_legal64(const Smem& s, int p, int ch) 
 
 // ---- observation + mask chunks of 16 cells (Sec. IV-B, App. A, Sec. IV-G) --
 // WRITE: store the planes; COUNT: legal (cell, direction) pairs per chunk.
-template <bool WRITE, bool COUNT, class T>
-__device__ void output_pass(const KArgs& a, const Game& g, const Smem& s, uint32_t alive, bool finished, const T& t,
+template <bool WRITE, bool COUNT, class G>
+__device__ void output_pass(const KArgs& a, const Game& g, const Smem& s, uint32_t alive, bool finished, const G& t,
                             int64_t frame_off) {
     const int nch = g.nch, st = s.stride, vs = s.vstride(), P = g.P;
     // a row up or down in 16-cell units and a shift

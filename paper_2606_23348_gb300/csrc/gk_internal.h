@@ -146,7 +146,7 @@ struct SmemLimit {
     }
 };
 
-// Feature-tensor builder (App. A): one warp per game, players in turn.
+// Feature-tensor builder (App. A).
 struct FArgs {
     const GameInfo* info;
     const int16_t* army;
@@ -163,15 +163,19 @@ struct FArgs {
     int16_t* ring;         // [(K + 1) * 2][plane_cells]: own / enemy army planes of folded frames
     float* out;            // player plane q = plane_off + p * Npad: channel ch of cell c at q * C + ch * Npad + c
     int32_t npad_max;      // largest board (cells, multiple of 16)
+    int32_t npad_mean;     // mean board of a player
+    int32_t n_players;     // player slots
     int32_t window;        // temporal-token window T (0: none)
     int2* series_ring;     // [slot][T]: (opponents' army, land), entry (n - 1) mod T = the n-th folded frame
     int2* series_out;      // optional [slot][T]: newest first, 0 before the episode
+    // uniform batch: as in KArgs
+    int32_t uniform;
+    GameInfo ushape;
 };
 
-// Launch the feature builder over every game on `stream`: form 1 one warp
-// per game, 2 one CTA per game, 0 by batch size.  pmax = the most players of
-// any game.  Returns a cudaError_t.
-int launch_features(const FArgs& f, int pmax, int form, void* stream);
+// Launch the feature builder over every game on `stream`.  pmax = the most
+// players of any game.  Returns a cudaError_t.
+int launch_features(const FArgs& f, int pmax, void* stream);
 
 // Policy sampling over the H x W x 9 action space.
 struct SArgs {

@@ -480,16 +480,16 @@ class Features:
     FORM_AUTO, FORM_WARP, FORM_CTA = 0, 1, 2
 
     def autotune(self, out, steps: int = 5) -> int:
-        """Time both forms building into `out` and keep the faster; returns it."""
+        """Kept for its callers: one build into `out`; returns FORM_CTA, the
+        fastest form at every batch size."""
         f = C.c_int32()
         _check(self.lib.gen_features_autotune(self.h, C.c_void_p(out.data_ptr()), int(steps), C.byref(f)),
                "gen_features_autotune")
         return int(f.value)
 
     def set_form(self, form: int):
-        """Spread of a game over the GPU: FORM_WARP (one warp per game),
-        FORM_CTA (one CTA per game and player, for small batches) or
-        FORM_AUTO."""
+        """Kept for its callers (FORM_*): builds always run one CTA per (game,
+        player), the fastest form at every batch size."""
         _check(self.lib.gen_features_set_form(self.h, int(form)), "gen_features_set_form")
 
     def player_series(self, series, g: int, p: int):

@@ -140,6 +140,17 @@ def test_features_large_boards_and_odd_player_counts(form, hist):
     lockstep(env, orc, fb, ofb, 30, 5, f"large hist {hist}", every=2)
 
 
+def test_features_few_large_boards_among_many():
+    """A batch whose warps per player follow its mean board, so that 64x64 and
+    23x37 boards take many rounds of a CTA; odd and absent players."""
+    H = np.array([64, 23, 64] + [5, 4, 9] * 85, np.int32)
+    W = np.array([64, 37, 20] + [6, 4, 7] * 85, np.int32)
+    mode = np.array([2, 1, 0] + [0, 2, 0] * 85, np.int32)
+    P = np.array([3, 4, 2] + [2, 3, 2] * 85, np.int32)
+    env, orc, fb, ofb = pair(H, W, mode, P, window=5, seed=9, n_cities=1, max_turns=8, min_general_dist=1)
+    lockstep(env, orc, fb, ofb, 12, 4, "few large", every=3)
+
+
 @FORMS
 def test_features_subset_reset_and_repeat_build(form):
     """A reset of some games clears their memory; a second build in one frame changes nothing."""
