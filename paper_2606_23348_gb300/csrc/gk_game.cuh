@@ -525,6 +525,8 @@ __device__ __forceinline__ void castle_guarantee(const KArgs& a, const Game& g, 
     }
 }
 
+__device__ __forceinline__ bool wide_rows(const Game& g) { return g.W > 32 || g.H > 32; }
+
 // ---- map generator (Sec. IV-A) ----------------------------------------------
 // Mountains, castles and taken cells are row-major bitsets while the map is
 // made; the cells' bytes are written once at the end, with the passable-
@@ -536,7 +538,13 @@ __device__ __forceinline__ void castle_guarantee(const KArgs& a, const Game& g, 
 // each, cells as bits until the end), 2,004 -> 419 us with BFS spacing and the
 // castle guarantee (see RowSet; 608 MB of state and outputs need 90 us).
 // SPAWN: with the options of the launch (a.spawn_*, a.castle_radius).
-template <int LW, bool SPAWN>
+// ROW_BITS: the word of a row bitset, 32 for boards of up to 32 rows and
+// columns, else 64; 0: by the game.  Launches of one shape know it, and
+// without the 64-bit rows' code the 32-bit rows keep more in registers (reset
+// of 65,536 24x24 games with BFS spacing and the castle guarantee: 388 -> 349
+// us; in a batch of both kinds, two generators would take turns in the
+// instruction cache: 8,192 mixed games 380 -> 430 us).
+template <int LW, bool SPAWN, int ROW_BITS>
 __device__ __forceinline__ void generate_body(const KArgs& a, const Game& g, const Smem& s, uint64_t gid,
                                              uint32_t epoch, const Grp<LW>& t) {
     const int N = g.N, W = g.W, P = g.P, nw = g.nw;
@@ -571,7 +579,7 @@ __device__ __forceinline__ void generate_body(const KArgs& a, const Game& g, con
     const int dmax = SPAWN ? a.spawn_dmax : 0;
     int my_gpos = -1;  // lane p holds player p's general
     bool carve = true;
-    const bool narrow_rows = g.W <= 32 && g.H <= 32;
+    const bool narrow_rows = ROW_BITS ? ROW_BITS == 32 : !wide_rows(g);
     if (SPAWN && a.spawn_bfs) {
         const int r = narrow_rows ? place_generals_bfs<uint32_t, 32 / LW>(g, mtn, kgen, dmax, t)
                                   : place_generals_bfs<uint64_t, 64 / LW>(g, mtn, kgen, dmax, t);
@@ -728,7 +736,7 @@ __device__ __forceinline__ void generate_body(const KArgs& a, const Game& g, con
 template <int LW, bool UNI, bool SPAWN>
 __device__ __noinline__ void generate(const KArgs& a, int gidx, char* warp_base, uint32_t geom, uint64_t gid,
                                      uint32_t epoch, int warp_lane) {
-    generate_body<LW, SPAWN>(a, game_of<UNI>(a, gidx), carve_geom(warp_base, geom), gid, epoch, Grp<LW>(warp_lane));
+    generate_body<LW, SPAWN, 0>(a, game_of<UNI>(a, gidx), carve_geom(warp_base, geom), gid, epoch, Grp<LW>(warp_lane));
 }
 
 // ---- one move on lane 0 (Sec. IV-D, IV-E) ----------------------------------
@@ -1417,7 +1425,7 @@ __device__ __forceinline__ Game group_game(Game g) {
 // generator returning, 132.5 us so; with the spawn options compiled in,
 // 185.7 us returning and 136.6 us so).
 // sc: the counters with the frame and epoch of the new state.
-template <int LW, bool UNI, bool SPAWN>
+template <int LW, bool UNI, bool SPAWN, int ROW_BITS>
 __device__ __noinline__ void new_map(const KArgs& a, int gidx, char* warp_base, uint32_t geom, int warp_lane,
                                      uint32_t frame, uint32_t epoch, uint32_t invalid, uint32_t saturated, uint32_t err,
                                      float my_reward, uint32_t done) {
@@ -1425,7 +1433,7 @@ __device__ __noinline__ void new_map(const KArgs& a, int gidx, char* warp_base, 
     const Game g = group_game<LW>(game_of<UNI>(a, gidx));
     const Smem s = carve_geom(warp_base, geom);
     if (a.op != OP_STEP && a.do_outputs) zero_guards(g, s, t);  // the step has set them
-    generate_body<LW, SPAWN>(a, g, s, game_id_of<UNI>(a, gidx), epoch, t);
+    generate_body<LW, SPAWN, ROW_BITS>(a, g, s, game_id_of<UNI>(a, gidx), epoch, t);
     const uint32_t alive = (1u << g.P) - 1u;
     cell_pass<true>(g, s, false, false, t);
     int32_t act = 0;
@@ -1452,8 +1460,15 @@ __device__ __forceinline__ void run_game(const KArgs& a, const Smem& s, char* wa
                 s1 = *(reinterpret_cast<const uint4*>(sc) + 1);
                 s0.z += 1;
             }
-            new_map<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of(a), t.lane + t.shift, s0.y, s0.z, s1.y, s1.z,
-                             s1.w, 0.0f, 0u);
+            const uint32_t whole = geom ? geom : geom_of(a);
+            if constexpr (SPAWN && UNI) {
+                if (wide_rows(g))
+                    new_map<LW, UNI, SPAWN, 64>(a, gidx, warp_base, whole, t.lane + t.shift, s0.y, s0.z, s1.y, s1.z, s1.w, 0.0f, 0u);
+                else
+                    new_map<LW, UNI, SPAWN, 32>(a, gidx, warp_base, whole, t.lane + t.shift, s0.y, s0.z, s1.y, s1.z, s1.w, 0.0f, 0u);
+            } else {
+                new_map<LW, UNI, SPAWN, 0>(a, gidx, warp_base, whole, t.lane + t.shift, s0.y, s0.z, s1.y, s1.z, s1.w, 0.0f, 0u);
+            }
             return;
         }
     }
@@ -1495,8 +1510,18 @@ __device__ __forceinline__ void run_game(const KArgs& a, const Smem& s, char* wa
                 if (a.auto_reset) {
                     epoch += 1;
                     if constexpr (!MULTI) {
-                        new_map<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of(a), t.lane + t.shift, frame + 1,
-                                         epoch, invalid, saturated, err, my_reward, done);
+                        const uint32_t whole = geom ? geom : geom_of(a);
+                        if constexpr (SPAWN && UNI) {
+                            if (wide_rows(g))
+                                new_map<LW, UNI, SPAWN, 64>(a, gidx, warp_base, whole, t.lane + t.shift, frame + 1, epoch, invalid,
+                                                            saturated, err, my_reward, done);
+                            else
+                                new_map<LW, UNI, SPAWN, 32>(a, gidx, warp_base, whole, t.lane + t.shift, frame + 1, epoch, invalid,
+                                                            saturated, err, my_reward, done);
+                        } else {
+                            new_map<LW, UNI, SPAWN, 0>(a, gidx, warp_base, whole, t.lane + t.shift, frame + 1, epoch, invalid,
+                                                       saturated, err, my_reward, done);
+                        }
                         return;
                     } else {
                         generate<LW, UNI, SPAWN>(a, gidx, warp_base, geom ? geom : geom_of(a),
