@@ -457,7 +457,7 @@ int gen_set_lane_groups(gen_env *env, int mode);
  * from an atomic counter and carve their shared memory per item; 0 (default)
  * = one launch of a CTA per game for small batches (up to 27 x the SM count
  * games, 40 x in four buckets or fewer), else 2 for batches of more than four
- * buckets, else 1.  The work list's
+ * buckets (three or four: up to 320 x the SM count games), else 1.  The work list's
  * counter belongs to the environment: order its calls on one stream.
  * GEN_ERR_BAD_ARG for NULL env or a form outside 0..2. */
 int gen_set_batch_form(gen_env *env, int form);

@@ -286,14 +286,19 @@ int launch_one(const Bucket& b, const KArgs& a, void* stream, const char* what) 
 // launch per size bucket (buckets after the first run on side streams forked
 // from and joined back into `stream`) or one work-list launch.
 // The work-list form serves batches of several buckets.  By default it takes
-// batches of more than four buckets: there the per-bucket launches are many
-// and small (mixed 32,768 games, 15 buckets: 136 against 131 M frames/s per
-// frame, resident 173 against 167 M), while a few large buckets overlap
-// well on the forked streams (ragged 131,072 games, 4 buckets: 428 against
-// 419 M, resident 627 against 606 M).
+// batches of more than four buckets, and of three or four up to 320 games
+// per SM: there the per-bucket launches are small and their tails and event
+// joins show, while a few large buckets overlap well on the forked streams
+// (1v1 games of 15..30 a side, four buckets, us per frame with the work list
+// and without: 32,768 games 73 and 79, 49,152 106 and 109, 65,536 139 and 137,
+// 131,072 271 and 257; 16-frame rollouts of 32,768 776 and 822; 20,000 2v2
+// games of 18..30 a side, three buckets, 88 and 98; 30,000 1v1 games of
+// 20..24 a side, two buckets, 65 and 62).
 bool use_worklist(const gen_env* e) {
     if (e->buckets.size() < 2 || !e->d_items[0] || e->batch_form == 1) return false;
-    return e->batch_form == 2 || e->buckets.size() > 4;
+    if (e->batch_form == 2) return true;
+    const size_t nb = e->buckets.size();
+    return nb > 4 || (nb > 2 && e->G <= 320 * gk::sm_count());
 }
 
 template <class Fill>

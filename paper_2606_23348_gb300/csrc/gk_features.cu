@@ -29,8 +29,6 @@
 // 2,613 us, 1,000 30x30 free-for-all games 255 against 319 us.
 #include <cuda_runtime.h>
 
-#include <atomic>
-
 #include <algorithm>
 #include <cstdint>
 
@@ -588,15 +586,6 @@ __global__ void __launch_bounds__(1024) k_features(const FArgs f, int pmax) {
 
 int launch_features(const FArgs& f, int pmax, void* stream) {
     if (f.n_games <= 0) return 0;
-    static std::atomic<int> sm_count{0};  // of the first device used: only the launch shape depends on it
-    int sms = sm_count.load(std::memory_order_relaxed);
-    if (sms == 0) {
-        int dev = 0, n = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        sms = n > 0 ? n : 1;
-        sm_count.store(sms, std::memory_order_relaxed);
-    }
     // Warps per player and chunks of 128 cells per warp at a time (32 warps of
     // an SM run at once at 62 registers).  A batch that fits gets a warp per
     // chunk of the largest board, or, where only that fits, a warp per two
@@ -606,7 +595,7 @@ int launch_features(const FArgs& f, int pmax, void* stream) {
     const int stage = item_stage_bytes(f.hist);
     const int fit = (227 * 1024 - cta_head_bytes(f.npad_max)) / stage;
     const int largest = (f.npad_max + 127) >> 7, mean = (f.npad_mean + 127) >> 7;
-    const int64_t room = 32 * (int64_t)sms;
+    const int64_t room = 32 * (int64_t)sm_count();
     int warps = mean, items = 1;
     if (f.n_players * (int64_t)largest <= room) {
         warps = largest;

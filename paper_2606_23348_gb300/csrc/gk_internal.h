@@ -239,6 +239,9 @@ int worklist_shape(bool multi, int* cta_smem, int* ctas);
 // take items until the list is done.  Returns a cudaError_t.
 int launch_worklist(const KArgs& a, const WArgs& w, int cta_smem, int ctas, void* stream);
 
+// SMs of the first device used: only launch shapes depend on it.
+int sm_count();
+
 // Launch the step kernel with `warps_per_cta` games per CTA on `stream`.
 // Returns a cudaError_t value.
 int launch_step(const KArgs& a, int warps_per_cta, int max_ctas, void* stream);

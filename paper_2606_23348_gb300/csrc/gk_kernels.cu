@@ -200,7 +200,6 @@ int launch_groups(const KArgs& a, int lw, bool multi, bool spawn, int fixed_warp
     return launch_chained(f, dim3(blocks), dim3(32 * warps), smem, st, a);
 }
 
-// SMs of the first device used: only launch shapes depend on it
 int sm_count() {
     static std::atomic<int> count{0};
     int sms = count.load(std::memory_order_relaxed);
@@ -256,7 +255,10 @@ int launch_step(const KArgs& a, int warps_per_cta, int max_ctas, void* stream) {
     const int wcap = warps_per_cta > 0 ? warps_per_cta : 1;  // the fixed shape must fit too
     int per_warp = 1;
     const bool spawn = has_spawn_options(a);
-    if (small && multi && !spawn && a.npad_max <= kQuadMaxCells && 4 * wcap * a.warp_smem <= 227 * 1024)
+    // four per warp from 32 games per SM on (16 frames of 24x24 1v1 games:
+    // 4,096 games 137 us with four, 127 us with two; 6,144 166 and 172; 8,192
+    // 199 and 238)
+    if (small && multi && !spawn && a.npad_max <= kQuadMaxCells && a.n_items >= 32 * sms && 4 * wcap * a.warp_smem <= 227 * 1024)
         per_warp = 4;
     else if (small && a.npad_max <= kPairMaxCells && 2 * wcap * a.warp_smem <= 227 * 1024)
         per_warp = 2;

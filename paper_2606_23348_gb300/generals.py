@@ -366,7 +366,8 @@ class GeneralsEnv:
         """How a batch of several size buckets launches: BATCH_BUCKETS (one
         launch per bucket), BATCH_WORKLIST (one persistent work-list launch)
         or BATCH_AUTO (one launch of a CTA per game for small batches, the work
-        list for larger ones of more than four buckets)."""
+        list for larger ones of more than four buckets, or of three or four
+        and not very large)."""
         _check(self.lib.gen_set_batch_form(self.h, int(form)), "gen_set_batch_form")
 
     def set_sample_form(self, form: int):
