@@ -426,8 +426,12 @@ int build_buckets(gen_env* e) {
     std::vector<int> order((size_t)e->G);
     for (int g = 0; g < e->G; ++g) order[(size_t)g] = g;
     auto key = [&](int g) { return game_class(e->h_info[(size_t)g]); };
-    // largest class first (it finishes last), then game id
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return key(x) > key(y); });
+    // the class with the most work per game first, cells times players (it
+    // finishes last), then game id
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+        const auto a = key(x), b = key(y);
+        return std::make_pair(a.first * a.second, a) > std::make_pair(b.first * b.second, b);
+    });
     e->buckets.clear();
     for (int i = 0; i < e->G;) {
         const auto k = key(order[(size_t)i]);
