@@ -1250,34 +1250,30 @@ __device__ int32_t policy_pass(const KArgs& a, const Game& g, const Smem& s, uin
     }
     int32_t action = 0;
     if (my_lane >= 0 && !finished && ((alive >> t.lane) & 1u)) {
-        for (int c = my_lane * cpl; c < nch; ++c) {
-            const uint32_t n = s.cnt[t.lane * nch + c];
-            if (my_rank >= n) {
-                my_rank -= n;
-                continue;
-            }
-            const uint64_t m = chunk_legal64(s, t.lane, c);
-            uint32_t x = (uint32_t)m;
-            int bit = 0;
-            const uint32_t nlo = __popc(x);
-            if (my_rank >= nlo) {
-                my_rank -= nlo;
-                x = (uint32_t)(m >> 32);
-                bit = 32;
-            }
-#pragma unroll
-            for (int w = 16; w >= 1; w >>= 1) {
-                const uint32_t cw = __popc(x & ((1u << w) - 1u));
-                if (my_rank >= cw) {
-                    my_rank -= cw;
-                    x >>= w;
-                    bit += w;
-                }
-            }
-            const int d = bit & 3;
-            action = (c * 16 + (bit >> 2)) * 9 + (my_half ? 5 + d : 1 + d);
-            break;
+        // the chunk first, so that the players' lanes part only in this loop
+        const uint8_t* cnt = s.cnt + t.lane * nch;
+        int c = my_lane * cpl;
+        for (uint32_t n = cnt[c]; my_rank >= n; n = cnt[++c]) my_rank -= n;
+        const uint64_t m = chunk_legal64(s, t.lane, c);
+        uint32_t x = (uint32_t)m;
+        int bit = 0;
+        const uint32_t nlo = __popc(x);
+        if (my_rank >= nlo) {
+            my_rank -= nlo;
+            x = (uint32_t)(m >> 32);
+            bit = 32;
         }
+#pragma unroll
+        for (int w = 16; w >= 1; w >>= 1) {
+            const uint32_t cw = __popc(x & ((1u << w) - 1u));
+            if (my_rank >= cw) {
+                my_rank -= cw;
+                x >>= w;
+                bit += w;
+            }
+        }
+        const int d = bit & 3;
+        action = (c * 16 + (bit >> 2)) * 9 + (my_half ? 5 + d : 1 + d);
     }
     if (DIRECT && t.lane < g.P) a.next_actions[g.player_off + t.lane] = action;
     return action;
