@@ -182,7 +182,10 @@ __global__ void __launch_bounds__(256, 4) k_team(const KArgs a) {
 }
 
 // Warps per game: the first and enough others to write the outputs (16-cell
-// chunks of every player) in about two rounds; fewer, down to two, when the
+// chunks of every player) in about two rounds, one more while that asks for
+// at most 20 warps per SM (32 frames of 1v1 games with one more and without:
+// 700 of 24x24 107 and 109 us, 1,000 of 15x15 100 and 106; 64 frames of 1,024
+// 24x24 games 245 and 239 us); fewer, down to two, when the
 // games would not all run at once (64 registers: 32 warps per SM; 16 frames of
 // 1,024 mixed games: 157 us, with up to 48 warps per SM asked for 214 us).
 int launch_team(const KArgs& a, int sms, void* stream) {
@@ -193,7 +196,8 @@ int launch_team(const KArgs& a, int sms, void* stream) {
     const int e = limits[spawn].raise(&fn, 1, a.warp_smem);
     if (e != 0) return e;
     const int chunks = a.pmax * (a.npad_max >> 4);
-    int warps = 1 + std::min(7, (chunks + 63) / 64 + 1);
+    int warps = 1 + std::min(7, (chunks + 63) / 64);
+    if (warps < 8 && (int64_t)a.n_items * (warps + 1) <= (int64_t)20 * sms) ++warps;
     while (warps > 2 && (int64_t)a.n_items * warps > (int64_t)28 * sms) --warps;
     const int threads = 32 * warps;
     return launch_chained(f, dim3(a.n_items), dim3(threads), a.warp_smem, (cudaStream_t)stream, a);
