@@ -180,7 +180,8 @@ __device__ __forceinline__ uint64_t warp_incl64(uint64_t x, int lane) {
 //
 // Bound by instructions and L1 wavefronts (65,536 1v1 games of 24x24 at mid-
 // game, N(0, 2) logits; the sectors of the own cells' logits and the board
-// need 79 us): 270 -> 143.6 us, 1,531 -> 952 warp instructions per player,
+// need 79 us): 270 -> 143.6 us, 1,531 -> 952 warp instructions per player
+// (134 us in runs of four players per warp, below),
 // against a warp per player that staged the board, loaded each logit by
 // itself and summed and scanned every 32 cells; 1,000 such games 7.9 -> 7.4,
 // 8,192 mixed games of 20..40 a side 243 -> 51 us (shared memory for eight
@@ -248,9 +249,14 @@ __device__ __forceinline__ float warp_max_nan(float m) {
     return m;
 }
 
-// player p's action in game gidx, by one warp; list: its shared memory
+// the draw of player p
+__device__ __forceinline__ uint64_t player_draw(const SArgs& a, const GameInfo& gi, const GameScalars& sc, int p) {
+    return stream_out(hkey(a.seed, gi.game_id, sc.frame, (uint64_t)p), 7);
+}
+
+// player p's action in game gidx from its draw d, by one warp; list: its shared memory
 __device__ __forceinline__ int32_t sample_player(const SArgs& a, const GameInfo& gi, const GameScalars& sc, int p,
-                                                 uint16_t* list, int lane) {
+                                                 uint64_t d, uint16_t* list, int lane) {
     const uint4* owner = reinterpret_cast<const uint4*>(a.owner + gi.cell_off);
     const uint32_t p4 = 0x01010101u * (uint32_t)p;
     int n = 0;
@@ -310,7 +316,6 @@ __device__ __forceinline__ int32_t sample_player(const SArgs& a, const GameInfo&
     }
     const uint64_t incl = warp_incl64(mine, lane);
     const uint64_t S = __shfl_sync(kAll, incl, 31);
-    const uint64_t d = stream_out(hkey(a.seed, gi.game_id, sc.frame, (uint64_t)p), 7);
     const uint64_t r = __umul64hi(d, S);
     const unsigned hit = __ballot_sync(kAll, incl > r);
     if (hit == 0u) return 0;  // S = 0: only when every legal logit is -inf (outside the documented domain)
@@ -399,7 +404,7 @@ __device__ __forceinline__ void sample_slot(const SArgs& a, int gidx, int p, cha
     if (p >= gi.P) return;
     const GameScalars sc = a.scal[gidx];
     uint16_t* list = reinterpret_cast<uint16_t*>(smem + (size_t)wid * list_bytes(a.npad_max));
-    const int32_t action = sample_player(a, gi, sc, p, list, lane);
+    const int32_t action = sample_player(a, gi, sc, p, player_draw(a, gi, sc, p), list, lane);
     if (lane == 0) a.actions[gi.player_off + p] = action;
 }
 __global__ void __launch_bounds__(32 * kSlotWarps, 36 / kSlotWarps) k_sample_slots(const SArgs a, int pmax) {
@@ -409,6 +414,31 @@ __global__ void __launch_bounds__(32 * kSlotWarps, 36 / kSlotWarps) k_sample_slo
     const unsigned item = blockIdx.x * kSlotWarps + wid;
     const int gidx = (int)(item / (unsigned)pmax), p = (int)item - gidx * pmax;
     if (gidx < a.n_games) sample_slot(a, gidx, p, smem, wid, lane);
+}
+// The same for large batches: `per` consecutive (game, player) items per warp,
+// whose draws are hashed side by side, a lane each (a hundred instructions
+// for all of them), and whose indexes are divided once.
+__global__ void __launch_bounds__(32 * kSlotWarps, 36 / kSlotWarps) k_sample_runs(const SArgs a, int pmax, int per) {
+    chain_entry();
+    extern __shared__ __align__(16) char smem[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint16_t* list = reinterpret_cast<uint16_t*>(smem + (size_t)wid * list_bytes(a.npad_max));
+    const unsigned item = (blockIdx.x * kSlotWarps + wid) * (unsigned)per + lane;
+    const int my_g = (int)(item / (unsigned)pmax), my_p = (int)item - my_g * pmax;
+    uint64_t my_d = 0;
+    if (lane < per && my_g < a.n_games) my_d = player_draw(a, sample_game(a, my_g), a.scal[my_g], my_p);
+#pragma unroll 1
+    for (int i = 0; i < per; ++i) {
+        const int gidx = __shfl_sync(kAll, my_g, i), p = __shfl_sync(kAll, my_p, i);
+        const uint64_t d = __shfl_sync(kAll, my_d, i);
+        if (gidx >= a.n_games) return;
+        const GameInfo gi = sample_game(a, gidx);
+        if (p >= gi.P) continue;
+        const GameScalars sc = a.scal[gidx];
+        const int32_t action = sample_player(a, gi, sc, p, d, list, lane);
+        if (lane == 0) a.actions[gi.player_off + p] = action;
+        __syncwarp();  // the list is reused
+    }
 }
 // The sampler and the expanded mask in one launch: per game, CTAs of four
 // players and one CTA for its mask.  The sampler waits on latency and the
@@ -439,6 +469,16 @@ int launch_sample(const SArgs& a, int pmax, void* stream) {
                               std::max(mask_smem, per * list_bytes(a.npad_max)), st, a, ctas_per_game);
     }
     const int64_t items = (int64_t)a.n_games * pmax;
+    // runs for batches of one shape (every item is a player) of many waves:
+    // 65,536 24x24 1v1 games 141.5 us with one item per warp, 136.6 with two,
+    // 134.3 with four; 16,384 games 39.9, 39.0 and 41.7; 4,000 games 11.5 and 11.9
+    const int64_t per_sm = items / sm_count();
+    const int per = !a.uniform || per_sm < 160 ? 1 : per_sm < 512 ? 2 : 4;
+    if (per > 1) {
+        const int64_t warps = (items + per - 1) / per;
+        return launch_chained(k_sample_runs, dim3((unsigned)((warps + kSlotWarps - 1) / kSlotWarps)),
+                              dim3(32 * kSlotWarps), kSlotWarps * list_bytes(a.npad_max), st, a, pmax, per);
+    }
     return launch_chained(k_sample_slots, dim3((unsigned)((items + kSlotWarps - 1) / kSlotWarps)), dim3(32 * kSlotWarps),
                           kSlotWarps * list_bytes(a.npad_max), st, a, pmax);
 }

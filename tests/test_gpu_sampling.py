@@ -147,6 +147,32 @@ def test_sampling_uniform_batch_extreme_logits(H, W, mode, P, G):
         assert torch.equal(alone, want)
 
 
+@pytest.mark.parametrize("G,mode,P", [(12163, 0, 2), (38915, 0, 2), (16219, 2, 3)])
+def test_sampling_runs_of_players_match_single_warps(G, mode, P):
+    """Uniform batches large enough for two or four players per warp, with a
+    last warp that is not full: the same games, split over environments that
+    are small enough for a player per warp, draw the same actions."""
+    import torch
+    from paper_2606_23348_gb300.generals import GeneralsEnv
+    kw = dict(batch=G, seed=6, n_cities=2, min_general_dist=2)
+    env = GeneralsEnv(5, 6, mode, P, **kw)
+    acts, out = env.new_actions(), env.new_outputs()
+    for f in range(12):
+        env.policy(3, acts)
+        env.step(acts, out)
+    gen = torch.Generator(device="cuda").manual_seed(8)
+    logits = torch.randn(int(env.layout.plane_cells) * 9, generator=gen, device="cuda") * 2
+    got = env.sample_actions(logits, 77)
+    st = env.read_state()
+    npad, part = int(env.npad[0]), 4096
+    for g0 in range(0, G, part):
+        n = min(part, G - g0)
+        small = GeneralsEnv(5, 6, mode, P, **dict(kw, batch=n, game_id_base=g0))
+        small.write_state(*(x[g0 * npad:(g0 + n) * npad] for x in st[:3]), st[3][g0:g0 + n])
+        want = small.sample_actions(logits[g0 * P * npad * 9:(g0 + n) * P * npad * 9].clone(), 77)
+        assert torch.equal(got[g0 * P:(g0 + n) * P], want), f"games {g0}.."
+
+
 @FORMS
 def test_sampling_large_territories(form):
     """Planted boards where one player owns most of a large board (hundreds of
