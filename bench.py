@@ -39,29 +39,23 @@ MAP_SEED = 1
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch
 # from one ncu capture, valid only for the kernel source with this hash: the
-# step kernel on the default workload's own 65,536 games (a one-pass capture
-# of one launch); the sampler on 16,384 games, scaled by the games it
-# processes (traffic grows in proportion).  Writes still dirty in the L2
+# step kernel and the sampler on 32,768 games, scaled by the games they process
+# (traffic grows in proportion).  Writes still dirty in the L2
 # when a launch ends are not in its DRAM count.
-NCU_TRAFFIC = {"kernel_sha1": "8302ad1d807f", "bytes_per_launch": 153810432.0 + 555577088.0,
-               "warp_inst_per_launch": 118105197.0, "captured": "65,536 games (the bench's own launch)",
-               "games": 65536}
+NCU_TRAFFIC = {"kernel_sha1": "b8bc4f67495f", "bytes_per_launch": 2 * (76900864.0 + 243619840.0),
+               "warp_inst_per_launch": 2 * 46636038.0, "captured": "32,768 games (x2)", "games": 65536}
 SM_COUNT, SCHEDULERS_PER_SM = 152, 4  # one warp instruction per scheduler and clock
-SAMPLE_NCU = {"kernel_sha1": "515d4f95a9c0", "bytes_per_launch": 4 * (133577216.0 + 3892480.0),
-              "warp_inst_per_launch": 4 * 50199088.0, "captured": "16,384 games (x4)", "games": 65536}
-# DRAM bytes of one frame of the ragged and mixed workloads, each in the form
-# that the default batch rule picks (per-bucket launches for the four ragged
-# buckets, summed; one work-list launch for the fifteen mixed buckets)
-ROLLOUT_NCU = {"kernel_sha1": "8302ad1d807f",
-               "1v1-131072-ragged15to30": {"form": "plain_buckets", "bytes_per_frame":
-                                           (30479872.0 + 145809408.0 + 139023104.0 + 5467136.0)
-                                           + (51041792.0 + 455997184.0 + 426810112.0 + 3328.0)},
-               "mixed-32768-sides20to40": {"form": "plain_worklist", "bytes_per_frame": 128557824.0 + 867469568.0}}
-FEATURE_NCU_TRAFFIC = {"kernel_sha1": "8af7d765f60a", "bytes_per_launch": 8 * (356319488.0 + 1554689024.0),
+SAMPLE_NCU = {"kernel_sha1": "85a5401c9388", "bytes_per_launch": 2 * (252385280.0 + 3618304.0),
+              "warp_inst_per_launch": 2 * 60473766.0, "captured": "32,768 games (x2)", "games": 65536}
+# DRAM bytes of one frame of the mixed workload in the form that the default
+# batch rule picks (one work-list launch, captured on 16,384 games, x2)
+ROLLOUT_NCU = {"kernel_sha1": "b8bc4f67495f",
+               "mixed-32768-sides20to40": {"form": "plain_worklist", "bytes_per_frame": 2 * (61724672.0 + 395919616.0)}}
+FEATURE_NCU_TRAFFIC = {"kernel_sha1": "183088f4da03", "bytes_per_launch": 8 * (351835648.0 + 1545319168.0),
                        "captured": "8,192 games (x8)", "games": 65536}
 
 
-def issue_roofline(launch_ms: float, G: int, clk, rec=None, source="gk_kernels.cu") -> dict | None:
+def issue_roofline(launch_ms: float, G: int, clk, rec=None, source="gk_game.cuh") -> dict | None:
     """An issue-bound kernel's second roofline: warp instructions per launch
     (ncu smsp__inst_executed.sum on the captured case, scaled by games) over
     the launch time, against SMs x schedulers x the SM clock sampled during
@@ -80,7 +74,7 @@ def issue_roofline(launch_ms: float, G: int, clk, rec=None, source="gk_kernels.c
             "source": f"ncu smsp__inst_executed.sum, {rec['captured']}; peak at the sampled {mhz} MHz"}
 
 
-def kernel_sha1(name: str = "gk_kernels.cu") -> str:
+def kernel_sha1(name: str = "gk_game.cuh") -> str:
     p = os.path.join(ROOT, "paper_2606_23348_gb300", "csrc", name)
     return hashlib.sha1(open(p, "rb").read()).hexdigest()[:12]
 
@@ -824,7 +818,7 @@ def sampler_record(args, G: int, K: int, rank: int = 0, clk=None) -> dict:
                          "algorithmic_bytes_per_launch": nbytes, "launch_ms": samp_ms,
                          "sector_bytes_per_launch": sector_bytes,
                          "frac_of_sector_bytes": sector_bytes / (samp_ms * 1e-3) / 1e9 / peak,
-                         "kernel": "k_sample_cta (H x W x 9 policy sampling, a CTA per game)"},
+                         "kernel": "k_sample_slots (H x W x 9 policy sampling, a warp per player)"},
             "issue_roofline": None}  # needs the clocks of the timed region: the caller adds it
 
 
@@ -1025,11 +1019,9 @@ def _graph_us(fn, T: int, stream) -> float:
 
 
 def run_forms_sweep(args, rank, world, local):
-    """Per-launch device time of every sampler form (warp per game, CTA per
-    game, CTA per player) and both feature-builder forms (warp per game, CTA
-    per player) on the default game shape (1v1 24x24) from 512 to 65,536
-    games, at mid-game (256 frames of the benchmark policy), each form
-    replayed as a CUDA graph of launches; and, at the self-play batch (512
+    """Per-launch device time of the sampler and the feature builder on the
+    default game shape (1v1 24x24) from 512 to 65,536 games, at mid-game (256
+    frames of the benchmark policy), each replayed as a CUDA graph of launches; and, at the self-play batch (512
     games), the sampler, step and feature launches alone and as a frame.
     Feature builds are timed as (step + build) - step, every build the first
     of its frame (the memory fold, the history ring full)."""
@@ -1060,20 +1052,13 @@ def run_forms_sweep(args, rank, world, local):
             sampled = env.new_actions()
             fb.build(x, tok)
             torch.cuda.synchronize()
-            row = {"games": G, "sampler_us": {}, "features_us": {}}
-            for form, name in ((1, "warp_per_game"), (2, "cta_per_game"), (3, "cta_per_player")):
-                env.set_sample_form(form)
-                row["sampler_us"][name] = _graph_us(lambda: env.sample_actions(logits, POLICY_SEED, sampled), T,
-                                                    stream)
+            row = {"games": G}
+            row["sampler_us"] = _graph_us(lambda: env.sample_actions(logits, POLICY_SEED, sampled), T, stream)
             # a build folds the frame into the players' memory once per frame:
             # timed as (step + build) - step, so that every build is a frame's first
             step_us = _graph_us(lambda: env.step_policy(acts, out, POLICY_SEED, acts), T, stream)
-            for form, name in ((1, "warp_per_game"), (2, "cta_per_player")):
-                fb.set_form(form)
-                row["features_us"][name] = _graph_us(lambda: (env.step_policy(acts, out, POLICY_SEED, acts),
-                                                              fb.build(x, tok)), T, stream) - step_us
-            env.set_sample_form(0)
-            fb.set_form(0)
+            row["features_us"] = _graph_us(lambda: (env.step_policy(acts, out, POLICY_SEED, acts),
+                                                    fb.build(x, tok)), T, stream) - step_us
             if G == 512:
                 frame = {"sample_us": _graph_us(lambda: env.sample_actions(logits, POLICY_SEED, sampled), T, stream),
                          "step_us": _graph_us(lambda: env.step(sampled, out), T, stream)}
@@ -1086,7 +1071,7 @@ def run_forms_sweep(args, rank, world, local):
             torch.cuda.empty_cache()
     if rank == 0:
         print(json.dumps({
-            "metric": "us per launch by form and batch size (sampler, feature builder)", "value": None,
+            "metric": "us per launch by batch size (sampler, feature builder)", "value": None,
             "unit": "us", "n_gpus": world, "higher_is_better": False, "vs_baseline": None,
             "dtype": "f32 logits and features, int16 state",
             "data": "synthetic (seeded counter-hash maps, N(0, 2) logits, 256 policy frames)",

@@ -1,7 +1,8 @@
 // Device code of the step kernels (instantiated by gk_kernels.cu, per frame,
-// gk_rollout.cu, multi-frame, and gk_worklist.cu): one group of lanes advances one Generals.io
-// game -- a warp, or for two-player games on small boards a half (two games
-// per warp) or, in multi-frame launches, a quarter of one (four per warp).
+// gk_rollout.cu, multi-frame, gk_worklist.cu and gk_team.cu): one group of
+// lanes advances one Generals.io game -- a warp, or for two-player games on
+// small boards a half (two games per warp) or, in multi-frame launches, a
+// quarter of one (four per warp); in small batches the warps of a CTA.
 //
 // Per game and step (paper Section IV) the group
 //   1. stages the board (int16 armies, int8 owners, int8 terrain) in shared
@@ -9,18 +10,18 @@
 //   2. resolves the players' moves one after another on its first lane
 //      (Sec. IV-D, IV-E), with a group-wide pass for the land transfer of a
 //      captured general;
-//   3. applies growth (Sec. IV-C) while ballots turn the board into 32-cell
-//      bitsets (ownership per player, army >= 2) and reductions total the
-//      armies;
+//   3. applies growth (Sec. IV-C) while dot products turn the board into
+//      bitsets (ownership per player, army >= 2) and total lands and armies;
 //   4. decides termination and reward (Sec. III) and regenerates finished
 //      games (Sec. IV-A);
-//   5. dilates the (team) ownership bitsets into fog-of-war visibility with
+//   5. widens the (team) ownership bitsets by a column to either side with
 //      word shifts (Sec. IV-B);
-//   6. expands bitsets and board bytes into 16-cell observation and mask
-//      chunks written with 128-bit streaming stores;
+//   6. joins the rows above and below into visibility and expands bitsets and
+//      board bytes into 16-cell observation and mask chunks written with
+//      128-bit streaming stores;
 //   7. optionally picks the next actions with the benchmark policy: legal
 //      (cell, direction) counts per chunk, a group scan to find the chunk, a
-//      scan over its 16 cells to find the cell.
+//      bisection of its legal moves to find the pair.
 //
 // Terrain bytes carry the cell type in bits 0-1 and, in bits 2-5, whether
 // the neighbour up / down / left / right exists and is not a mountain.  The
@@ -536,7 +537,8 @@ __device__ __forceinline__ bool wide_rows(const Game& g) { return g.W > 32 || g.
 // Instructions bound it.  Resets of 65,536 24x24 games: 314.6 -> 204.7 us with
 // the plain generator (castles a batch of draws at a time instead of a batch
 // each, cells as bits until the end), 2,004 -> 419 us with BFS spacing and the
-// castle guarantee (see RowSet; 608 MB of state and outputs need 90 us).
+// castle guarantee (see RowSet; 608 MB of state and outputs need 90 us), with
+// the step's newer passes 184 and 388 us.
 // SPAWN: with the options of the launch (a.spawn_*, a.castle_radius).
 // ROW_BITS: the word of a row bitset, 32 for boards of up to 32 rows and
 // columns, else 64; 0: by the game.  Launches of one shape know it, and
@@ -729,8 +731,8 @@ __device__ __forceinline__ void generate_body(const KArgs& a, const Game& g, con
     t.sync();
 }
 
-// Out-of-line entry point of a new map inside a multi-frame launch: it takes
-// plain arguments and rebuilds the game and shared-memory views itself, so
+// Out-of-line entry point of a new map inside a multi-frame launch or a CTA
+// per game: it takes plain arguments and rebuilds the game and shared-memory views itself, so
 // that the step kernel never materialises those structures in local memory
 // for a call it rarely makes.
 template <int LW, bool UNI, bool SPAWN>
@@ -1413,8 +1415,7 @@ __device__ __forceinline__ Game group_game(Game g) {
 }
 
 // The rest of a per-frame launch for a game that gets a new map (create,
-// reset, a finished game) or new passable-neighbour bits: the map, the
-// frame's end, the state stored.  Nothing returns to the step, so the step
+// reset, a finished game): the map, the frame's end, the state stored.  Nothing returns to the step, so the step
 // kernel keeps no value alive across a call: with the generator as a call
 // that returned, its registers set the spills of the frames without a reset
 // (65,536 1v1 games on 24x24: 135.5 us per launch with the earlier, smaller
@@ -1556,7 +1557,7 @@ __device__ __forceinline__ void run_game(const KArgs& a, const Smem& s, char* wa
 // game of the launch has the launch's shape (uniform batches).
 // Register budget: 64 per thread (4 CTAs of 8 warps per SM) for the per-frame
 // form; the multi-frame form keeps more state live across frames and runs
-// best with 85 (3 CTAs).
+// best with 80 (3 CTAs).
 template <bool MULTI, bool SPAWN, int LW, bool UNI>
 __global__ void __launch_bounds__(256, MULTI ? 3 : 4) k_generals(const KArgs a) {
     chain_entry();
