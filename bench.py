@@ -818,7 +818,7 @@ def sampler_record(args, G: int, K: int, rank: int = 0, clk=None) -> dict:
                          "algorithmic_bytes_per_launch": nbytes, "launch_ms": samp_ms,
                          "sector_bytes_per_launch": sector_bytes,
                          "frac_of_sector_bytes": sector_bytes / (samp_ms * 1e-3) / 1e9 / peak,
-                         "kernel": "k_sample_slots (H x W x 9 policy sampling, a warp per player)"},
+                         "kernel": "k_sample_runs (H x W x 9 policy sampling, a warp per player, four in turn)"},
             "issue_roofline": None}  # needs the clocks of the timed region: the caller adds it
 
 
