@@ -51,7 +51,7 @@ SAMPLE_NCU = {"kernel_sha1": "85a5401c9388", "bytes_per_launch": 2 * (252385280.
 # batch rule picks (one work-list launch, captured on 16,384 games, x2)
 ROLLOUT_NCU = {"kernel_sha1": "b8bc4f67495f",
                "mixed-32768-sides20to40": {"form": "plain_worklist", "bytes_per_frame": 2 * (61724672.0 + 395919616.0)}}
-FEATURE_NCU_TRAFFIC = {"kernel_sha1": "183088f4da03", "bytes_per_launch": 8 * (351835648.0 + 1545319168.0),
+FEATURE_NCU_TRAFFIC = {"kernel_sha1": "5c7cfd276cd5", "bytes_per_launch": 8 * (351877376.0 + 1545384448.0),
                        "captured": "8,192 games (x8)", "games": 65536}
 
 

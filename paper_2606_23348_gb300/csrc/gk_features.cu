@@ -471,8 +471,9 @@ __device__ __forceinline__ void stage_item(const FArgs& f, const HdrState& y, in
 // player's visibility bitset and the others the scoreboard (a warp per
 // player); then warp w takes the player's 128-cell chunks w, w + warps, ...
 // ITEMS at a time.
-template <int ITEMS>
-__global__ void __launch_bounds__(1024) k_features(const FArgs f, int pmax) {
+// LEAN: 56 registers, for 36 warps per SM instead of 32.
+template <int ITEMS, bool LEAN>
+__global__ void __maxnreg__(LEAN ? 56 : 64) k_features(const FArgs f, int pmax) {
     extern __shared__ __align__(16) char smem[];
     chain_entry();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -586,29 +587,39 @@ __global__ void __launch_bounds__(1024) k_features(const FArgs f, int pmax) {
 
 int launch_features(const FArgs& f, int pmax, void* stream) {
     if (f.n_games <= 0) return 0;
-    // Warps per player and chunks of 128 cells per warp at a time (32 warps of
-    // an SM run at once at 62 registers).  A batch that fits gets a warp per
-    // chunk of the largest board, or, where only that fits, a warp per two
-    // (512 24x24 1v1 games' self-play frame 37.2 against 39.5 us); larger ones
-    // a warp per chunk of the mean board, larger boards taking several rounds
-    // (2,048 mixed games of 20..40 a side 300 us, for the largest board 394).
+    // Warps per player and chunks of 128 cells per warp at a time.  A batch whose
+    // CTAs fit the GPU at once, by warps and by shared memory, gets a warp per
+    // chunk of the largest board, or, where only that fits, a warp per two (200
+    // 40x40 1v1 games: step and build 34.4 against 39.4 us; where two do not fit
+    // they lose, 600 24x24 games 45.9 against 37.2); larger ones a warp per chunk
+    // of the mean board, larger boards taking several rounds (2,048 mixed games
+    // of 20..40 a side 300 us, for the largest board 394).  The lean kernel runs
+    // where an SM holds a CTA more of it (512 24x24 1v1 games' self-play frame
+    // 35.8 against 37.3 us, 1,024 games 58.0 against 61.8; 2,048 mixed games,
+    // whose CTAs of eight warps it holds no more of, 309 against 302).
     const int stage = item_stage_bytes(f.hist);
-    const int fit = (227 * 1024 - cta_head_bytes(f.npad_max)) / stage;
-    const int largest = (f.npad_max + 127) >> 7, mean = (f.npad_mean + 127) >> 7;
-    const int64_t room = 32 * (int64_t)sm_count();
-    int warps = mean, items = 1;
-    if (f.n_players * (int64_t)largest <= room) {
+    const int fit = std::min(32, (227 * 1024 - cta_head_bytes(f.npad_max)) / stage);
+    const int largest = std::min(fit, (f.npad_max + 127) >> 7), half = (((f.npad_max + 127) >> 7) + 1) / 2;
+    auto ctas = [&](int warps, int items, int warps_per_sm) {  // per SM, 1 KB of its shared memory kept for each
+        return std::min(warps_per_sm / warps, 228 * 1024 / (cta_bytes(f.npad_max, f.hist, warps, items) + 1024));
+    };
+    auto fits = [&](int warps, int items, int warps_per_sm) {
+        return f.n_players <= ctas(warps, items, warps_per_sm) * (int64_t)sm_count();
+    };
+    int warps = std::max(1, std::min(fit, (f.npad_mean + 127) >> 7)), items = 1;
+    if (fits(largest, 1, 36)) {
         warps = largest;
-    } else if (f.n_players * (int64_t)((largest + 1) / 2) <= room && 2 * ((largest + 1) / 2) <= fit) {
-        warps = (largest + 1) / 2;
+    } else if (2 * half <= fit && fits(half, 2, 32)) {
+        warps = half;
         items = 2;
     }
-    warps = std::max(1, std::min(std::min(32, fit / items), warps));
     const int smem = cta_bytes(f.npad_max, f.hist, warps, items);
-    void (*const fn)(FArgs, int) = items == 1 ? k_features<1> : k_features<2>;
+    const bool lean = items == 1 && ctas(warps, 1, 36) > ctas(warps, 1, 32);
+    void (*const fn)(FArgs, int) = items == 2 ? k_features<2, false> : lean ? k_features<1, true> : k_features<1, false>;
     static SmemLimit limit;
-    static const void* const fns[2] = {(const void*)k_features<1>, (const void*)k_features<2>};
-    const int e = limit.raise(fns, 2, smem);
+    static const void* const fns[3] = {(const void*)k_features<1, true>, (const void*)k_features<1, false>,
+                                       (const void*)k_features<2, false>};
+    const int e = limit.raise(fns, 3, smem);
     if (e != 0) return e;
     return launch_chained(fn, dim3((unsigned)((int64_t)f.n_games * pmax)), dim3(32 * warps), smem, (cudaStream_t)stream,
                           f, pmax);

@@ -151,6 +151,15 @@ def test_features_few_large_boards_among_many():
     lockstep(env, orc, fb, ofb, 12, 4, "few large", every=3)
 
 
+@pytest.mark.parametrize("H,W,games", [(11, 11, 300), (31, 33, 20), (40, 40, 200)], ids=["1-lean", "1", "2"])
+def test_features_chunks_per_warp_and_registers(H, W, games):
+    """Each form of the kernel: one chunk per warp, where fewer registers let an
+    SM hold more CTAs (1 warp) or not (8), and two (more CTAs of 13 warps than fit)."""
+    env, orc, fb, ofb = pair([H] * games, [W] * games, [1] * games, [2] * games, window=3, seed=6, n_cities=1,
+                             max_turns=4)
+    lockstep(env, orc, fb, ofb, 6, 3, f"forms {H}x{W}", every=2)
+
+
 @FORMS
 def test_features_subset_reset_and_repeat_build(form):
     """A reset of some games clears their memory; a second build in one frame changes nothing."""
